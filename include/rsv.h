@@ -402,10 +402,10 @@ rsv_status rsv_draw_momenta(rsv_ctx* ctx, uint64_t seed, uint64_t series, uint64
 rsv_status rsv_ff_exp(rsv_ctx* ctx, const double* t, double* out, double* out2, int64_t n,
                       void* stream);
 /* rsv_fp64_exp: the exponential of the FP64 path's force and energies
- * (exp_tab): Tang's table-driven method, t = k ln2/64 + r, |r| <= ln2/128,
- * e^t = 2^(k div 64) 2^((k mod 64)/64) (1 + p(r)), p the degree-5 Taylor
- * polynomial of e^r - 1, the table 2^(j/64) rounded to double; |t| >= 512
- * falls back to CUDA's exp.  t, out: [n] device FP64.  n >= 0 and non-NULL
+ * (exp_neg, at -t): Tang's table-driven method in 64-bit fixed point,
+ * t = k ln2/1024 + r, e^t = 2^(k div 1024) 2^((k mod 1024)/1024) (1 + p(r)), p
+ * the Taylor polynomial of e^r - 1 to degree 4, rounded once; |t| >= 128 falls
+ * back to CUDA's exp.  t, out: [n] device FP64.  n >= 0 and non-NULL
  * pointers when n > 0, else RSV_EINVAL. */
 rsv_status rsv_fp64_exp(rsv_ctx* ctx, const double* t, double* out, int64_t n, void* stream);
 

@@ -192,53 +192,90 @@ __device__ __forceinline__ ff ff_exp(ff t, const float2* tab)
 }
 
 // ---------------------------------------------------------------------------
-// exp in FP64 for the FP64 trajectory kernel, table-driven after P. T. P. Tang
-// ("Table-driven implementation of the exponential function in IEEE
-// floating-point arithmetic", ACM TOMS 15, 1989): a = k ln2/64 + r with k the
-// integer nearest to 64 a/ln2 and |r| <= ln2/128 (ln2/64 split in a head of 32
-// significant bits, so that k times it is exact, and a tail), and
-//   e^a = 2^(k div 64) 2^((k mod 64)/64) (1 + p(r)),
-// p the Taylor polynomial of e^r - 1 to degree 5 (remainder < 4e-17 for
-// |r| <= ln2/128): 10 FP64 instructions.  kExp2Tab holds 2^(j/64) rounded to
-// double (computed to 200 bits).  |a| >= 512 takes exp (the scaling by
-// 2^(k div 64) through the exponent field assumes a normal result).
+// e^{-x} in FP64 without the FP64 pipe.  That pipe issues 2 lanes per cycle and
+// SM here (0.62 T instructions/s), the integer units 64, and the FP64 kernels
+// are bound by it, so the exponential is evaluated in 64-bit fixed point on the
+// integer units.  Table-driven after P. T. P. Tang ("Table-driven
+// implementation of the exponential function in IEEE floating-point
+// arithmetic", ACM TOMS 15, 1989): with a = -x in units of 2^-56 (|a| < 128),
+//   a = k ln2/1024 + r, 0 <= r < ln2/1024 (k floored from the top bits of a;
+//   r in units of 2^-66, ln2/1024 to 98 bits),
+//   e^a = 2^(k div 1024) T (1 + p),  T = 2^((k mod 1024)/1024) to 63 bits,
+//   p = r + r^2/2 + r^3 (1/6 + r/24)   (remainder r^5/120 < 2^-59),
+// the product rounded once, to nearest, into the result's mantissa: within
+// 0.61 ulp of e^a (0.51 away from x = 0; the truncation of a to 2^-56 is the
+// excess), against ~1.1 ulp of the form on FP64 instructions with a 64-entry
+// table that it replaced.  About 55 integer instructions and no FP64 ones, where
+// that form took 10 of the 18 FP64 instructions of a leapfrog step's site.
+// |x| >= 128, NaN, and the one or two arguments in a million whose floor or
+// last carry is ambiguous take CUDA's exp.
+// The table is the products of two 32-entry ones, 2^(i/32) and 2^(j/1024) in
+// units of 2^-63 (rounded from 60 decimal digits).
 // ---------------------------------------------------------------------------
-constexpr int kExpTabN = 64;
-static __constant__ double kExp2Tab[kExpTabN] = {
-    0x1.0000000000000p+0, 0x1.02c9a3e778061p+0, 0x1.059b0d3158574p+0, 0x1.0874518759bc8p+0,
-    0x1.0b5586cf9890fp+0, 0x1.0e3ec32d3d1a2p+0, 0x1.11301d0125b51p+0, 0x1.1429aaea92de0p+0,
-    0x1.172b83c7d517bp+0, 0x1.1a35beb6fcb75p+0, 0x1.1d4873168b9aap+0, 0x1.2063b88628cd6p+0,
-    0x1.2387a6e756238p+0, 0x1.26b4565e27cddp+0, 0x1.29e9df51fdee1p+0, 0x1.2d285a6e4030bp+0,
-    0x1.306fe0a31b715p+0, 0x1.33c08b26416ffp+0, 0x1.371a7373aa9cbp+0, 0x1.3a7db34e59ff7p+0,
-    0x1.3dea64c123422p+0, 0x1.4160a21f72e2ap+0, 0x1.44e086061892dp+0, 0x1.486a2b5c13cd0p+0,
-    0x1.4bfdad5362a27p+0, 0x1.4f9b2769d2ca7p+0, 0x1.5342b569d4f82p+0, 0x1.56f4736b527dap+0,
-    0x1.5ab07dd485429p+0, 0x1.5e76f15ad2148p+0, 0x1.6247eb03a5585p+0, 0x1.6623882552225p+0,
-    0x1.6a09e667f3bcdp+0, 0x1.6dfb23c651a2fp+0, 0x1.71f75e8ec5f74p+0, 0x1.75feb564267c9p+0,
-    0x1.7a11473eb0187p+0, 0x1.7e2f336cf4e62p+0, 0x1.82589994cce13p+0, 0x1.868d99b4492edp+0,
-    0x1.8ace5422aa0dbp+0, 0x1.8f1ae99157736p+0, 0x1.93737b0cdc5e5p+0, 0x1.97d829fde4e50p+0,
-    0x1.9c49182a3f090p+0, 0x1.a0c667b5de565p+0, 0x1.a5503b23e255dp+0, 0x1.a9e6b5579fdbfp+0,
-    0x1.ae89f995ad3adp+0, 0x1.b33a2b84f15fbp+0, 0x1.b7f76f2fb5e47p+0, 0x1.bcc1e904bc1d2p+0,
-    0x1.c199bdd85529cp+0, 0x1.c67f12e57d14bp+0, 0x1.cb720dcef9069p+0, 0x1.d072d4a07897cp+0,
-    0x1.d5818dcfba487p+0, 0x1.da9e603db3285p+0, 0x1.dfc97337b9b5fp+0, 0x1.e502ee78b3ff6p+0,
-    0x1.ea4afa2a490dap+0, 0x1.efa1bee615a27p+0, 0x1.f50765b6e4540p+0, 0x1.fa7c1819e90d8p+0,
+constexpr int kExpN = 1024;
+typedef unsigned long long u64;
+static __constant__ u64 kExpHi[32] = {
+    0x8000000000000000ull, 0x82cd8698ac2ba1d7ull, 0x85aac367cc487b15ull, 0x88980e8092da8527ull,
+    0x8b95c1e3ea8bd6e7ull, 0x8ea4398b45cd53c0ull, 0x91c3d373ab11c336ull, 0x94f4efa8fef70961ull,
+    0x9837f0518db8a96full, 0x9b8d39b9d54e5539ull, 0x9ef5326091a111aeull, 0xa27043030c496819ull,
+    0xa5fed6a9b15138eaull, 0xa9a15ab4ea7c0ef8ull, 0xad583eea42a14ac6ull, 0xb123f581d2ac2590ull,
+    0xb504f333f9de6484ull, 0xb8fbaf4762fb9ee9ull, 0xbd08a39f580c36bfull, 0xc12c4cca66709456ull,
+    0xc5672a115506daddull, 0xc9b9bd866e2f27a3ull, 0xce248c151f8480e4ull, 0xd2a81d91f12ae45aull,
+    0xd744fccad69d6af4ull, 0xdbfbb797daf23755ull, 0xe0ccdeec2a94e111ull, 0xe5b906e77c8348a8ull,
+    0xeac0c6e7dd24392full, 0xefe4b99bdcdaf5cbull, 0xf5257d152486cc2cull, 0xfa83b2db722a033aull,
 };
-__device__ __forceinline__ double exp_tab(double a, const double* tab)
+static __constant__ u64 kExpLo[32] = {
+    0x8000000000000000ull, 0x8016302f17467628ull, 0x802c6436d0e04f51ull, 0x80429c17d77c18edull,
+    0x8058d7d2d5e5f6b1ull, 0x806f17687707a7b0ull, 0x80855ad965e88b84ull, 0x809ba2264dada76aull,
+    0x80b1ed4fd999ab6cull, 0x80c83c56b50cf780ull, 0x80de8f3b8b85a0afull, 0x80f4e5ff089f763full,
+    0x810b40a1d81406d4ull, 0x81219f24a5baa59dull, 0x813801881d886f7cull, 0x814e67cceb90502dull,
+    0x8164d1f3bc030773ull, 0x817b3ffd3b2f2e47ull, 0x8191b1ea15813bfdull, 0x81a827baf7838b78ull,
+    0x81bea1708dde6056ull, 0x81d51f0b8557ec1dull, 0x81eba08c8ad45370ull, 0x820225f44b55b33cull,
+    0x8218af4373fc25ecull, 0x822f3c7ab205c89bull, 0x8245cd9ab2cec048ull, 0x825c62a423d13f0cull,
+    0x8272fb97b2a5894cull, 0x828998760d01faf3ull, 0x82a0393fe0bb0ca8ull, 0x82b6ddf5dbc35907ull,
+};
+// Fill tab[kExpN] (shared memory, the whole block; the caller synchronises).
+__device__ __forceinline__ void exp_table(u64* tab)
 {
-    const long long ab = __double_as_longlong(a);
-    if (((ab >> 52) & 0x7ff) >= 1032) return exp(a);  // |a| >= 512
-    const double sh = 0x1.8p52;  // adding it rounds to an integer
-    const double ks = fma(a, 0x1.71547652b82fep+6, sh);  // 64/ln2
-    const int k = (int)(__double_as_longlong(ks) - __double_as_longlong(sh));
-    const double kd = ks - sh;
-    double r = fma(-kd, 0x1.62e42fee00000p-7, a);  // head of ln2/64
-    r = fma(-kd, 0x1.a39ef35793c76p-39, r);          // its tail
-    double q = fma(r, 0x1.1111111111111p-7, 0x1.5555555555555p-5);  // 1/120, 1/24
-    q = fma(r, q, 0x1.5555555555555p-3);                               // 1/6
-    q = fma(r, q, 0.5);
-    const double p = fma(r * r, q, r);
-    const double t = tab[k & (kExpTabN - 1)];
-    const double e = fma(t, p, t);
-    return __longlong_as_double(__double_as_longlong(e) + ((long long)(k >> 6) << 52));
+    for (int i = threadIdx.x; i < kExpN; i += blockDim.x) {
+        const u64 a = kExpHi[i >> 5], b = kExpLo[i & 31];
+        const u64 hi = __umul64hi(a, b), lo = a * b;
+        tab[i] = (hi << 1) + (lo >> 63) + ((lo >> 62) & 1);  // the product in units of 2^-63, rounded
+    }
+}
+static __device__ __noinline__ double exp_slow(double a) { return exp(a); }
+// e^{-x / 2^SH} (SH = 0 or 1; the halving is exact)
+template <int SH = 0>
+__device__ __forceinline__ double exp_neg(double x, const u64* tab)
+{
+    const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
+    // |a| = M 2^(6 - sh - 62), M the 53-bit significand at bit 62
+    const int sh = 1029 + SH - (int)((xh >> 20) & 0x7ffu);  // < 0: |a| >= 128, inf, NaN
+    const u64 M = (((u64)((xh & 0xfffffu) | 0x100000u) << 32) | xl) << 10;
+    const unsigned s63 = (unsigned)sh < 63u ? (unsigned)sh : 63u;
+    const u64 m56 = M >> s63;
+    const u64 A = (int)xh < 0 ? m56 : 0ull - m56;  // a in units of 2^-56
+    // k = floor(a 1024/ln2) from the top 32 bits of a and 1024/ln2 in units of 2^-20
+    const int k = __mulhi((int)(A >> 32), 0x5c551d94) >> 12;
+    // ln2/1024 = (0xb17217f7d1cf7a - 0x54361c4c 2^-32) 2^-66
+    const u64 R = (A << 10) - (u64)((long long)k * 0xb17217f7d1cf7aLL) +
+                  (u64)(long long)__mulhi(k, 0x54361c4c);
+    const unsigned rr = (unsigned)(R >> 24);  // r in units of 2^-42
+    const u64 r2 = (u64)rr * rr;              // r^2 in units of 2^-84
+    const unsigned c = __umulhi((unsigned)(r2 >> 32), rr);         // r^3, 2^-62
+    const unsigned w = __umulhi(rr, 174763u) + 0x2aaaaaabu;        // 1/6 + r/24, 2^-32
+    const u64 P = R + (r2 >> 19) + (__umulhi(rr, (unsigned)R << 8) >> 18) +
+                  ((u64)__umulhi(c, w) << 4);                      // p, 2^-66
+    const u64 T = tab[k & (kExpN - 1)];
+    const unsigned Th = (unsigned)(T >> 32), Tl = (unsigned)T;
+    const unsigned Ph = (unsigned)(P >> 32), Pl = (unsigned)P;
+    const u64 tp = (u64)Th * Ph + __umulhi(Th, Pl) + __umulhi(Tl, Ph);  // T p, 2^-65
+    const u64 m = T + (tp >> 2);
+    // a negative r, a carry out of m (bit 63 is set otherwise) or |a| >= 128
+    if (((int)(R >> 32) | (int)~(unsigned)(m >> 32) | sh) < 0)
+        return exp_slow(SH ? -0.5 * x : -x);
+    const u64 v = (m >> 11) + ((m >> 10) & 1);
+    return __longlong_as_double((long long)(v + ((u64)(unsigned)((k >> 10) + 1022) << 52)));
 }
 
 // ---------------------------------------------------------------------------

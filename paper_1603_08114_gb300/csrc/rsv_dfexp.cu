@@ -1,7 +1,7 @@
 // rsv_dfexp.cu -- the exponentials of the trajectory kernels, exposed for
 // tests: the mixed path's double-float ff_exp (one double-float) and its
 // two-lane form ff2_exp (the end-of-trajectory statistics), and the FP64
-// path's table-driven exp_tab, evaluated at given arguments.  Not steps of
+// path's exp_neg, evaluated at given arguments.  Not steps of
 // the method; the tests compare them with exp in FP64.
 #include <algorithm>
 #include <cstdint>
@@ -46,16 +46,16 @@ __global__ void __launch_bounds__(kDfThreads) k_ff_exp(const double* __restrict_
     }
 }
 
-// exp_tab (the FP64 trajectory kernel's exponential) at each argument.
-__global__ void __launch_bounds__(kDfThreads) k_exp_tab(const double* __restrict__ t, int64_t n,
+// e^t by exp_neg (the FP64 kernels' exponential) at each argument.
+__global__ void __launch_bounds__(kDfThreads) k_exp_neg(const double* __restrict__ t, int64_t n,
                                                         double* __restrict__ out)
 {
-    __shared__ double tab[kExpTabN];
-    if (threadIdx.x < kExpTabN) tab[threadIdx.x] = kExp2Tab[threadIdx.x];
+    __shared__ u64 tab[kExpN];
+    exp_table(tab);
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x)
-        out[i] = exp_tab(t[i], tab);
+        out[i] = exp_neg(-t[i], tab);
 }
 
 }  // namespace
@@ -87,8 +87,8 @@ extern "C" rsv_status rsv_fp64_exp(rsv_ctx* c, const double* t, double* out, int
     if (n == 0) return RSV_OK;
     if (!t || !out) return fail(RSV_EINVAL, "null t or out");
     const int grid = (int)std::min<int64_t>((n + kDfThreads - 1) / kDfThreads, 4 * (int64_t)c->num_sms);
-    k_exp_tab<<<grid, kDfThreads, 0, (cudaStream_t)stream>>>(t, n, out);
+    k_exp_neg<<<grid, kDfThreads, 0, (cudaStream_t)stream>>>(t, n, out);
     c->launches += 1;
     cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? RSV_OK : cuda_fail(e, "k_exp_tab");
+    return e == cudaSuccess ? RSV_OK : cuda_fail(e, "k_exp_neg");
 }

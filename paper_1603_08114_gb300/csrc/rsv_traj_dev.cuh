@@ -45,19 +45,6 @@ __device__ __forceinline__ void exchange(V first, V last, V& left_last, V& right
     right_first = lane == 31 ? (has_r ? er : last) : dn;
 }
 
-// Innovations e_j = x_{j+1} - phi x_j of one thread's run (xR = first x of the
-// next thread), with e = 0 at the segment's last active slot `la`.
-template <int J, typename V, bool EDGE>
-__device__ __forceinline__ void innovations(const V (&x)[J], V xR, V phi, int la, V (&e)[J])
-{
-#pragma unroll
-    for (int j = 0; j < J; ++j) {
-        const V nx = (j + 1 < J) ? x[j + 1] : xR;
-        e[j] = fma(-phi, x[j], nx);
-        if (EDGE && j == la) e[j] = V(0);
-    }
-}
-
 // Per-thread view of the bin being processed.
 struct View {
     int sid;     // segment id, -1 for an idle warp
