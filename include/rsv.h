@@ -86,8 +86,8 @@ int rsv_abi_version(void);
 rsv_status rsv_sync_status(rsv_ctx* ctx, void* stream);
 /* Fix the tiling of single-series trajectories (rsv_hmc_trajectory,
  * rsv_hmc_chain) and of plans created afterwards: `threads` per block
- * (multiple of 32; <= 256 FP64, <= 384 mixed), `sites_per_thread` (FP64: 4, 8,
- * 16, 28; mixed: 4, 8, 16, 20) and `tile` owned sites per tile of a series cut
+ * (multiple of 32; <= 256 FP64, <= 384 mixed), `sites_per_thread` (FP64: 1, 2,
+ * 4, 8, 16, 28; mixed: 4, 8, 16, 20) and `tile` owned sites per tile of a series cut
  * into tiles (tile + 2 (n_md + 1) + 3 <= threads * sites_per_thread, else the
  * call that uses it fails with RSV_EINVAL).  A single series no longer than
  * `tile` is kept whole (it then needs only T <= threads * sites_per_thread).

@@ -22,9 +22,9 @@ namespace rsv {
 
 namespace {
 
-const int kJ_fp64[] = {4, 8, 16, 28};
+const int kJ_fp64[] = {1, 2, 4, 8, 16, 28};
 const int kJ_mixed[] = {4, 8, 12, 16, 20};
-const int kNJ_fp64 = 4, kNJ_mixed = 5;
+const int kNJ_fp64 = 6, kNJ_mixed = 5;
 
 // mixed: (a, k) float2 + x0 (hi, lo) + p0 per site (+ dtau/m with a mass,
 // + the leverage v with leverage), the start state in j rows of
@@ -46,6 +46,24 @@ bool valid_j(bool mixed, int j)
     for (int i = 0; i < n; ++i)
         if (js[i] == j) return true;
     return false;
+}
+
+// Time in us of one FP64 trajectory of a single series as `bins` blocks of nt
+// threads with j sites each, n_force force evaluations, of which bps fit on an
+// SM.  A step is the longer of one warp's own latency (0.30 + 0.36 j) and the
+// SM's FP64 pipe, which all its warps share (0.50 + 0.0625 j per warp); a
+// launch's draws, energies and decision about 16 + 3 j.  Fitted to a sweep of
+// every shape (32 .. 256 threads, j = 1 .. 28) at T = 500 .. 2^18 and n_md = 10
+// .. 80, off by 10 % at most near the optimum: T = 2000, 50 steps 46 us (87 blocks of
+// 128 x 1) against 121 us (4 blocks of 192 x 4, the fewest sites in flight),
+// T = 30000, 50 steps 72 us (160 x 2) against 106 us (128 x 4).
+double fp64_cost(int64_t bins, int nt, int j, int n_force, int num_sms, int bps)
+{
+    const int64_t per = std::min<int64_t>(bps, (bins + num_sms - 1) / num_sms);
+    const int64_t waves = (bins + per * num_sms - 1) / (per * num_sms);
+    const double warps = (double)per * (nt / 32);
+    const double step = std::max(0.30 + 0.36 * j, 0.50 + 0.0625 * j * warps);
+    return waves * (16.0 + 3.0 * j + n_force * step) * (1.0 + 1e-6 * bins);
 }
 
 int ntmax(bool mixed, bool mass, int j) { return mixed ? mixed_max_threads(j, mass) : 256; }
@@ -139,6 +157,7 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                     if (bps < 1) continue;
                     const int64_t waves = (b + (int64_t)num_sms * bps - 1) / ((int64_t)num_sms * bps);
                     double cost = (double)waves * (double)cap * bps;
+                    if (!mixed) cost = fp64_cost(b, t, js[ji], (int)(K - 1), num_sms, bps);
                     // measured on the mixed kernel at T = 2^20 (fixed and
                     // per-step cost per block shape): J = 12 with ~600
                     // threads is the fastest, J = 20 close, J = 16 and 8
@@ -158,7 +177,7 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                     // trajectory in 4 waves, 288 x 20 0.449 ms in 5 (25 %
                     // more per site); a whole series keeps the smallest
                     // window (a tie-break toward more threads only)
-                    cost *= 1.0 + (b > 1 ? 1.0 : 1e-3) * (double)(tmax - t) / tmax;
+                    if (mixed) cost *= 1.0 + (b > 1 ? 1.0 : 1e-3) * (double)(tmax - t) / tmax;
                     if (cost < best) {
                         best = cost;
                         nt = t;

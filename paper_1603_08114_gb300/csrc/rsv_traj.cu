@@ -536,7 +536,7 @@ int blocks_per_sm(bool mixed, bool mass, bool lev, int j, int nt, size_t smem)
     if (mixed) {
         switch (j) { RSV_JM(4) RSV_JM(8) RSV_JM(12) RSV_JM(16) RSV_JM(20) default: return 0; }
     } else {
-        switch (j) { RSV_JD(4) RSV_JD(8) RSV_JD(16) RSV_JD(28) default: return 0; }
+        switch (j) { RSV_JD(1) RSV_JD(2) RSV_JD(4) RSV_JD(8) RSV_JD(16) RSV_JD(28) default: return 0; }
     }
 #undef RSV_JM
 #undef RSV_JD
@@ -565,6 +565,8 @@ cudaError_t launch_traj(const TrajArgs& a, const Plan& p, cudaStream_t st)
         }
     }
     switch (p.j) {
+        RSV_CASE(launch_fp64, 1)
+        RSV_CASE(launch_fp64, 2)
         RSV_CASE(launch_fp64, 4)
         RSV_CASE(launch_fp64, 8)
         RSV_CASE(launch_fp64, 16)
