@@ -104,9 +104,9 @@ rsv_status rsv_set_schedule(rsv_ctx* ctx, int threads, int sites_per_thread, int
  * The results are bit for bit those of the per-trajectory launches. */
 rsv_status rsv_set_persistent(rsv_ctx* ctx, int enable);
 /* rsv_set_wait_limit: the clock cycles (per SM) a device-side wait of the
- * persistent chain may spin before it gives up: it then records a timeout,
- * which rsv_sync_status() returns as RSV_ETIMEOUT, and the kernel ends (the
- * chain's results are invalid; the context stays usable).  0 restores the
+ * persistent chain or of rsv_mlp_train may spin before it gives up: it then
+ * records a timeout, which rsv_sync_status() returns as RSV_ETIMEOUT, and the
+ * kernel ends (the call's results are invalid; the context stays usable).  0 restores the
  * default, 2^31 cycles (about one second at 2 GHz); cycles < 0: RSV_EINVAL. */
 rsv_status rsv_set_wait_limit(rsv_ctx* ctx, int64_t cycles);
 /* rsv_chain_schedule: the block shape an rsv_hmc_chain call of this context

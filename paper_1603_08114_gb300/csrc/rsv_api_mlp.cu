@@ -74,11 +74,10 @@ rsv_status rsv_mlp_grad(rsv_ctx* c, const float* feat, const float* target, int6
     if (st != RSV_OK) return st;
     if (!params || !grad_out) return fail(RSV_EINVAL, "null argument");
     if ((st = mlp_common(c, feat, target, T, batch)) != RSV_OK) return st;
-    cudaError_t e = counted(c, launch_mlp_step, feat, target, T, const_cast<float*>(params),
-                            (float*)nullptr, (float*)nullptr, grad_out, c->extra.as<float>(),
-                            reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter),
-                            seed, step, (int64_t)1, 0.f, 0.f, 0.f, 0.f, batch, 0, loss_out,
-                            log_scale, (cudaStream_t)stream);
+    cudaError_t e = counted(c, launch_mlp_step, feat, target, T, const_cast<float*>(params), grad_out,
+                            c->extra.as<float>(),
+                            reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter), seed,
+                            step, batch, loss_out, log_scale, (cudaStream_t)stream);
     return e == cudaSuccess ? RSV_OK : cuda_fail(e, "mlp gradient kernel");
 }
 
@@ -93,17 +92,13 @@ rsv_status rsv_mlp_train(rsv_ctx* c, const float* feat, const float* target, int
     if (step0 < 0 || n_steps < 0) return fail(RSV_EINVAL, "negative step");
     if (!(lr > 0.f)) return fail(RSV_EINVAL, "lr must be > 0");
     if ((st = mlp_common(c, feat, target, T, batch)) != RSV_OK) return st;
-    for (int i = 0; i < n_steps; ++i) {
-        const uint64_t step = (uint64_t)(step0 + i);
-        cudaError_t e = counted(c, launch_mlp_step, feat, target, T, params, adam_m, adam_v,
-                                (float*)nullptr, c->extra.as<float>(),
-                                reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter),
-                                seed, step, (int64_t)(step + 1), lr, 0.9f, 0.999f, 1e-8f, batch, 1,
-                                loss_out ? loss_out + i : (float*)nullptr, log_scale,
-                                (cudaStream_t)stream);
-        if (e != cudaSuccess) return cuda_fail(e, "mlp step kernel");
-    }
-    return RSV_OK;
+    unsigned* cnt = reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter);
+    cudaError_t e = launch_mlp_train(feat, target, T, params, adam_m, adam_v, c->extra.as<float>(),
+                                     cnt, cnt + 2, seed, step0, n_steps, lr, batch, loss_out,
+                                     log_scale, capture_active(), c->num_sms, c->wait_limit,
+                                     c->ints.as<int>() + kStatus, &c->launches,
+                                     (cudaStream_t)stream);
+    return e == cudaSuccess ? RSV_OK : cuda_fail(e, "mlp training kernel");
 }
 
 rsv_status rsv_mlp_mass(rsv_ctx* c, const float* feat, int64_t T, const float* params,

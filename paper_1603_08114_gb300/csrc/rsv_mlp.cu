@@ -45,11 +45,6 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
     const uint32_t b = __bfloat16_as_ushort(__float2bfloat16_rn(hi));
     return a | (b << 16);
 }
-__device__ __forceinline__ float round_bf16(float x)
-{
-    return __bfloat162float(__float2bfloat16_rn(x));
-}
-
 // D = A(16x16, row) * B(16x8, col) + C, BF16 inputs, FP32 accumulate.
 __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
                                          uint32_t b1)
@@ -67,67 +62,98 @@ __device__ __forceinline__ float softplus_f(float z)
 }
 __device__ __forceinline__ float sigmoid_f(float z) { return 1.f / (1.f + expf(-z)); }
 
-// Shared parameter copies of one block.
-struct SParams {
-    float w1[NH * KP];  // BF16-rounded, K padded with zeros
-    float w2[NH * NH];  // BF16-rounded
+// Shared parameter copies of one block.  The BF16 matrices have rows of LD
+// entries (80 bytes): the eight rows of a fragment start in different banks and
+// each row on a 16-byte boundary, as ldmatrix wants.
+constexpr int LD = 40;
+struct __align__(16) SParams {
+    __nv_bfloat16 w1[NH * LD];   // W1[n][k], K padded with zeros
+    __nv_bfloat16 w2[NH * LD];   // W2[n][k]
+    __nv_bfloat16 w2t[NH * LD];  // W2[n][k] at [k][n], for the back-propagation
     float b1[NH], b2[NH], w3[NH];
     float b3;
 };
 
-__device__ void load_params(const float* __restrict__ P, SParams& s)
+// The block's copy of the parameters (through L2: the training kernel's blocks
+// update them during the launch); all loads of a thread are issued together.
+template <int THREADS>
+__device__ __forceinline__ void load_params(const float* __restrict__ P, SParams& s)
 {
-    for (int i = threadIdx.x; i < NH * KP; i += blockDim.x) {
-        const int n = i / KP, k = i % KP;
-        s.w1[i] = k < NF ? round_bf16(P[OFF_W1 + n * NF + k]) : 0.f;
+    constexpr int N = (NPARAM + THREADS - 1) / THREADS;
+    float v[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int e = threadIdx.x + i * THREADS;
+        v[i] = e < NPARAM ? __ldcg(P + e) : 0.f;
     }
-    for (int i = threadIdx.x; i < NH * NH; i += blockDim.x) s.w2[i] = round_bf16(P[OFF_W2 + i]);
-    for (int i = threadIdx.x; i < NH; i += blockDim.x) {
-        s.b1[i] = P[OFF_B1 + i];
-        s.b2[i] = P[OFF_B2 + i];
-        s.w3[i] = P[OFF_W3 + i];
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const int e = threadIdx.x + i * THREADS;
+        if (e < OFF_B1) {
+            s.w1[(e / NF) * LD + e % NF] = __float2bfloat16_rn(v[i]);
+        } else if (e < OFF_W2) {
+            s.b1[e - OFF_B1] = v[i];
+        } else if (e < OFF_B2) {
+            const int n = (e - OFF_W2) / NH, k = (e - OFF_W2) % NH;
+            s.w2[n * LD + k] = s.w2t[k * LD + n] = __float2bfloat16_rn(v[i]);
+        } else if (e < OFF_W3) {
+            s.b2[e - OFF_B2] = v[i];
+        } else if (e < OFF_B3) {
+            s.w3[e - OFF_W3] = v[i];
+        } else if (e < NPARAM) {
+            s.b3 = v[i];
+        }
     }
-    if (threadIdx.x == 0) s.b3 = P[OFF_B3];
+}
+// zero the padding columns of w1 (once per block)
+template <int THREADS>
+__device__ __forceinline__ void pad_params(SParams& s)
+{
+    for (int i = threadIdx.x; i < NH * (KP - NF); i += THREADS)
+        s.w1[(i / (KP - NF)) * LD + NF + i % (KP - NF)] = __float2bfloat16_rn(0.f);
 }
 
 // B fragment (16 x 8, "col") of a matrix stored as M[n][k] (row n, K
 // consecutive): element (k, n) = M[n0 + n][k0 + k].
-__device__ __forceinline__ void b_frag_nk(const float* M, int ld, int n0, int k0, uint32_t& b0,
+__device__ __forceinline__ void b_frag_nk(const __nv_bfloat16* M, int n0, int k0, uint32_t& b0,
                                           uint32_t& b1)
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const float* r = M + (n0 + g) * ld + k0;
-    b0 = pack_bf16(r[2 * t], r[2 * t + 1]);
-    b1 = pack_bf16(r[2 * t + 8], r[2 * t + 9]);
+    const uint32_t* r = reinterpret_cast<const uint32_t*>(M + (n0 + g) * LD + k0);
+    b0 = r[t];
+    b1 = r[t + 4];
 }
-// B fragment of a matrix stored as M[k][n]: element (k, n) = M[k0 + k][n0 + n].
-__device__ __forceinline__ void b_frag_kn(const float* M, int ld, int k0, int n0, uint32_t& b0,
-                                          uint32_t& b1)
+// A fragment (16 x 16, row) of a matrix stored as M[m][k]: (m, k) = M[m][k0 + k].
+__device__ __forceinline__ void a_frag_mk(const __nv_bfloat16* M, int k0, uint32_t (&a)[4])
 {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    b0 = pack_bf16(M[(k0 + 2 * t) * ld + n0 + g], M[(k0 + 2 * t + 1) * ld + n0 + g]);
-    b1 = pack_bf16(M[(k0 + 2 * t + 8) * ld + n0 + g], M[(k0 + 2 * t + 9) * ld + n0 + g]);
+    const uint32_t* r0 = reinterpret_cast<const uint32_t*>(M + g * LD + k0);
+    const uint32_t* r1 = reinterpret_cast<const uint32_t*>(M + (g + 8) * LD + k0);
+    a[0] = r0[t];
+    a[1] = r1[t];
+    a[2] = r0[t + 4];
+    a[3] = r1[t + 4];
 }
-// A fragment (16 x 16, row) of a matrix stored as M[m][k]: (m, k) = M[m0 + m][k0 + k].
-__device__ __forceinline__ void a_frag_mk(const float* M, int ld, int m0, int k0, uint32_t (&a)[4])
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&d)[4], const __nv_bfloat16* row)
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const float* r0 = M + (m0 + g) * ld + k0;
-    const float* r1 = M + (m0 + g + 8) * ld + k0;
-    a[0] = pack_bf16(r0[2 * t], r0[2 * t + 1]);
-    a[1] = pack_bf16(r1[2 * t], r1[2 * t + 1]);
-    a[2] = pack_bf16(r0[2 * t + 8], r0[2 * t + 9]);
-    a[3] = pack_bf16(r1[2 * t + 8], r1[2 * t + 9]);
+    const uint32_t p = (uint32_t)__cvta_generic_to_shared(row);
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(d[0]), "=r"(d[1]), "=r"(d[2]), "=r"(d[3])
+                 : "r"(p)
+                 : "memory");
 }
-// A fragment of the TRANSPOSE of M[k][m]: (m, k) = M[k0 + k][m0 + m].
-__device__ __forceinline__ void a_frag_t(const float* M, int ld, int m0, int k0, uint32_t (&a)[4])
+// A fragment (16 x 16) of the TRANSPOSE of M[k][m], 16 rows k: (m, k) = M[k][m0 + m].
+__device__ __forceinline__ void a_frag_t(const __nv_bfloat16* M, int m0, uint32_t (&a)[4])
 {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    a[0] = pack_bf16(M[(k0 + 2 * t) * ld + m0 + g], M[(k0 + 2 * t + 1) * ld + m0 + g]);
-    a[1] = pack_bf16(M[(k0 + 2 * t) * ld + m0 + g + 8], M[(k0 + 2 * t + 1) * ld + m0 + g + 8]);
-    a[2] = pack_bf16(M[(k0 + 2 * t + 8) * ld + m0 + g], M[(k0 + 2 * t + 9) * ld + m0 + g]);
-    a[3] = pack_bf16(M[(k0 + 2 * t + 8) * ld + m0 + g + 8],
-                     M[(k0 + 2 * t + 9) * ld + m0 + g + 8]);
+    const int lane = threadIdx.x & 31, tile = lane >> 3, r = lane & 7;
+    ldmatrix_x4_trans(a, M + ((tile >> 1) * 8 + r) * LD + m0 + (tile & 1) * 8);
+}
+// B fragments (16 x 8 each) of columns n0 .. n0+7 (b[0], b[1]) and n0+8 ..
+// n0+15 (b[2], b[3]) of a matrix stored as M[k][n], 16 rows k.
+__device__ __forceinline__ void b_frag_kn2(const __nv_bfloat16* M, int n0, uint32_t (&b)[4])
+{
+    const int lane = threadIdx.x & 31, tile = lane >> 3, r = lane & 7;
+    ldmatrix_x4_trans(b, M + ((tile & 1) * 8 + r) * LD + n0 + (tile >> 1) * 8);
 }
 // A fragment of a 16 x 32 activation held as C fragments c[ntile][4] (k-step kk).
 __device__ __forceinline__ void a_from_c(const float (&c)[4][4], int kk, uint32_t (&a)[4])
@@ -136,6 +162,17 @@ __device__ __forceinline__ void a_from_c(const float (&c)[4][4], int kk, uint32_
     a[1] = pack_bf16(c[2 * kk][2], c[2 * kk][3]);
     a[2] = pack_bf16(c[2 * kk + 1][0], c[2 * kk + 1][1]);
     a[3] = pack_bf16(c[2 * kk + 1][2], c[2 * kk + 1][3]);
+}
+// C fragments of a 16 x 32 activation into M[s][n] (BF16 pairs).
+__device__ __forceinline__ void store_c(const float (&c)[4][4], __nv_bfloat16* M)
+{
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt) {
+        *reinterpret_cast<uint32_t*>(M + g * LD + 8 * nt + 2 * t) = pack_bf16(c[nt][0], c[nt][1]);
+        *reinterpret_cast<uint32_t*>(M + (g + 8) * LD + 8 * nt + 2 * t) =
+            pack_bf16(c[nt][2], c[nt][3]);
+    }
 }
 
 // Site index of minibatch entry k of Adam step `step`: word k%4 of Philox
@@ -147,9 +184,9 @@ __device__ __forceinline__ int64_t batch_site(uint64_t seed, uint64_t step, int6
     return (int64_t)((hi * (uint64_t)T) >> 32);
 }
 
-// Forward of the 16 sites of this warp.  fs: [16][KP] BF16-rounded features
+// Forward of the 16 sites of this warp.  fs: [16][LD] features in BF16
 // (shared).  Outputs: a1, a2 in C-fragment form, z3 for rows g and g+8.
-__device__ __forceinline__ void mlp_forward(const SParams& sp, const float* fs, float (&a1)[4][4],
+__device__ __forceinline__ void mlp_forward(const SParams& sp, const __nv_bfloat16* fs, float (&a1)[4][4],
                                             float (&a2)[4][4], float& z3g, float& z3g8)
 {
     const int lane = threadIdx.x & 31, t = lane & 3;
@@ -157,11 +194,11 @@ __device__ __forceinline__ void mlp_forward(const SParams& sp, const float* fs, 
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
         uint32_t a[4];
-        a_frag_mk(fs, KP, 0, 16 * kk, a);
+        a_frag_mk(fs, 16 * kk, a);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
             uint32_t b0, b1;
-            b_frag_nk(sp.w1, KP, 8 * nt, 16 * kk, b0, b1);
+            b_frag_nk(sp.w1, 8 * nt, 16 * kk, b0, b1);
             mma_bf16(z1[nt], a, b0, b1);
         }
     }
@@ -181,7 +218,7 @@ __device__ __forceinline__ void mlp_forward(const SParams& sp, const float* fs, 
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
             uint32_t b0, b1;
-            b_frag_nk(sp.w2, NH, 8 * nt, 16 * kk, b0, b1);
+            b_frag_nk(sp.w2, 8 * nt, 16 * kk, b0, b1);
             mma_bf16(z2[nt], a, b0, b1);
         }
     }
@@ -205,9 +242,6 @@ __device__ __forceinline__ void mlp_forward(const SParams& sp, const float* fs, 
     z3g8 = pg8 + sp.b3;
 }
 
-// One minibatch: loss and gradient partials of this block; the last block to
-// arrive sums the partials in block order and (update != 0) takes an Adam
-// step of the FP32 master parameters.
 struct StepArgs {
     const float* feat;    // [T][NF] standardised features
     const float* target;  // [T]
@@ -216,8 +250,8 @@ struct StepArgs {
     float* adam_m;
     float* adam_v;
     float* grad_out;      // optional: the gradient of this batch [NPARAM]
-    float* partials;      // [gridDim.x][NPARAM + 1]
-    unsigned* counter;
+    float* partials;      // [batch / 64][NPARAM + 1]
+    unsigned* counter;    // arrival counter (step kernel) or grid barrier (training kernel)
     uint64_t seed, step;  // minibatch of Adam step `step`
     int64_t adam_t;       // 1-based Adam time of this step
     float lr, b1, b2, eps;
@@ -225,38 +259,70 @@ struct StepArgs {
     int update;
     float* loss_out;      // optional
     const float* log_scale;  // optional device scalar: log s
+    // training kernel: steps of this launch, the barrier's wait limit (clock
+    // cycles) and the status word that tells of a wait that ran out
+    int n_steps;
+    long long wait_limit;
+    int* status;
 };
 
-__global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
+// The features and targets of a warp's 16 sites of one minibatch, fetched into
+// registers: lane l holds elements l, l + 32, ... of the 16 x NF features, and
+// the site index and target of entry l & 15.
+struct Fetch {
+    float f[16 * NF / 32];
+    float y;
+};
+static_assert(16 * NF % 32 == 0, "whole lanes");
+__device__ __forceinline__ void fetch_sites(const StepArgs& A, uint64_t step, int64_t k0, Fetch& q)
 {
-    __shared__ SParams sp;
-    __shared__ float fs[4][16][KP];   // features of the warp's sites (BF16-rounded)
-    __shared__ float st_a1[4][16][NH];  // a1 (BF16-rounded) for dW2
-    __shared__ float st_d[4][16][NH];   // dz2, then dz1 (BF16-rounded)
-    __shared__ float gsum[NPARAM + 1];  // block gradient (+ loss in the last slot)
-    __shared__ int s_last;
+    const int lane = threadIdx.x & 31;
+    const int64_t site = batch_site(A.seed, step, k0 + (lane & 15), A.T);
+    q.y = A.target[site];
+#pragma unroll
+    for (int i = 0; i < 16 * NF / 32; ++i) {
+        const int e = lane + 32 * i;
+        q.f[i] = A.feat[__shfl_sync(0xffffffffu, site, e / NF) * NF + e % NF];
+    }
+}
+
+// The block's working memory (dynamic shared memory).
+struct __align__(16) StepSmem {
+    SParams sp;
+    __nv_bfloat16 fs[4][16 * LD];  // features of the warp's sites
+    __nv_bfloat16 a1[4][16 * LD];  // a1, for dW2
+    __nv_bfloat16 d[4][16 * LD];   // dz2, then dz1
+    float grad[4][NPARAM + 1];     // each warp's gradient (and loss, the last slot)
+};
+__device__ __forceinline__ void pad_features(StepSmem& S)
+{
+    for (int i = threadIdx.x; i < 4 * 16 * (KP - NF); i += blockDim.x)
+        S.fs[0][(i / (KP - NF)) * LD + NF + i % (KP - NF)] = __float2bfloat16_rn(0.f);
+}
+
+// Loss and gradient of one group of 64 minibatch sites (16 per warp) by a
+// block of 128 threads, into part[NPARAM + 1]: the warps' sums added in warp
+// order.  The parameters are in S.sp, the warp's sites in q; ends with the
+// block's stores to part issued (no barrier).
+__device__ __forceinline__ void mlp_group(StepSmem& S, const Fetch& q, const StepArgs& A, float ls,
+                                          float* __restrict__ part)
+{
+    const SParams& sp = S.sp;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-    load_params(A.params, sp);
-    for (int i = tid; i < NPARAM + 1; i += blockDim.x) gsum[i] = 0.f;
-    // gather this warp's 16 sites
-    const int64_t k0 = (int64_t)blockIdx.x * SITES_PER_BLOCK + warp * 16;
-    if (lane < 16) {
-        const int64_t site = batch_site(A.seed, A.step, k0 + lane, A.T);
-        for (int f = 0; f < KP; ++f)
-            fs[warp][lane][f] = f < NF ? round_bf16(A.feat[site * NF + f]) : 0.f;
+    __nv_bfloat16* fs = S.fs[warp];
+    __nv_bfloat16* st_a1 = S.a1[warp];
+    __nv_bfloat16* st_d = S.d[warp];
+    float* gr = S.grad[warp];
+#pragma unroll
+    for (int i = 0; i < 16 * NF / 32; ++i) {
+        const int e = lane + 32 * i;
+        fs[(e / NF) * LD + e % NF] = __float2bfloat16_rn(q.f[i]);
     }
-    __syncthreads();
+    __syncwarp();
     float a1[4][4], a2[4][4], z3g, z3g8;
-    mlp_forward(sp, &fs[warp][0][0], a1, a2, z3g, z3g8);
+    mlp_forward(sp, fs, a1, a2, z3g, z3g8);
     // loss gradient at rows g and g+8
-    float yg, yg8;
-    {
-        const int64_t sg = batch_site(A.seed, A.step, k0 + g, A.T);
-        const int64_t sg8 = batch_site(A.seed, A.step, k0 + g + 8, A.T);
-        yg = A.target[sg];
-        yg8 = A.target[sg8];
-    }
-    const float ls = A.log_scale ? *A.log_scale : 0.f;
+    const float yg = __shfl_sync(0xffffffffu, q.y, g), yg8 = __shfl_sync(0xffffffffu, q.y, g + 8);
     const float mg = softplus_f(z3g) + EPS_M, mg8 = softplus_f(z3g8) + EPS_M;
     const float lg = logf(mg) + ls - yg, lg8 = logf(mg8) + ls - yg8;
     const float invB = 1.f / (float)A.batch;
@@ -277,41 +343,27 @@ __global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
             pb2[nt][c] = dz2[nt][c] + dz2[nt][2 + c];
         }
     }
-    // sum over the 8 groups of the warp (rows), then one lane per column adds
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1) {
-                pw3[nt][c] += __shfl_xor_sync(0xffffffffu, pw3[nt][c], o);
-                pb2[nt][c] += __shfl_xor_sync(0xffffffffu, pb2[nt][c], o);
-            }
-    // stage a1 and dz2 (BF16-rounded) for the weight gradient of layer 2
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
-        const int n0 = 8 * nt + 2 * t;
-        st_a1[warp][g][n0] = round_bf16(a1[nt][0]);
-        st_a1[warp][g][n0 + 1] = round_bf16(a1[nt][1]);
-        st_a1[warp][g + 8][n0] = round_bf16(a1[nt][2]);
-        st_a1[warp][g + 8][n0 + 1] = round_bf16(a1[nt][3]);
-        st_d[warp][g][n0] = round_bf16(dz2[nt][0]);
-        st_d[warp][g][n0 + 1] = round_bf16(dz2[nt][1]);
-        st_d[warp][g + 8][n0] = round_bf16(dz2[nt][2]);
-        st_d[warp][g + 8][n0 + 1] = round_bf16(dz2[nt][3]);
-    }
+    // stage a1 and dz2 for the weight gradient of layer 2
+    store_c(a1, st_a1);
+    store_c(dz2, st_d);
     __syncwarp();
     // dW2[n][k] = sum_s dz2[s][n] a1[s][k]: M = n (2 tiles), N = k (4 tiles), K = 16 sites
-    float gw2[2][4][4] = {};
+    uint32_t b1f[2][4];
+    b_frag_kn2(st_a1, 0, b1f[0]);
+    b_frag_kn2(st_a1, 16, b1f[1]);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
         uint32_t a[4];
-        a_frag_t(&st_d[warp][0][0], NH, 16 * mt, 0, a);
+        a_frag_t(st_d, 16 * mt, a);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
-            uint32_t b0, b1;
-            b_frag_kn(&st_a1[warp][0][0], NH, 0, 8 * nt, b0, b1);
-            mma_bf16(gw2[mt][nt], a, b0, b1);
+            float gw[4] = {};
+            mma_bf16(gw, a, b1f[nt >> 1][2 * (nt & 1)], b1f[nt >> 1][2 * (nt & 1) + 1]);
+            const int n = 16 * mt + g, k = 8 * nt + 2 * t;
+            gr[OFF_W2 + n * NH + k] = gw[0];
+            gr[OFF_W2 + n * NH + k + 1] = gw[1];
+            gr[OFF_W2 + (n + 8) * NH + k] = gw[2];
+            gr[OFF_W2 + (n + 8) * NH + k + 1] = gw[3];
         }
     }
     // da1 = dz2 W2 (A = dz2 rows = sites; B(k=n, n=j) = W2[n][j])
@@ -319,131 +371,232 @@ __global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
 #pragma unroll
     for (int kk = 0; kk < 2; ++kk) {
         uint32_t a[4];
-        a[0] = pack_bf16(dz2[2 * kk][0], dz2[2 * kk][1]);
-        a[1] = pack_bf16(dz2[2 * kk][2], dz2[2 * kk][3]);
-        a[2] = pack_bf16(dz2[2 * kk + 1][0], dz2[2 * kk + 1][1]);
-        a[3] = pack_bf16(dz2[2 * kk + 1][2], dz2[2 * kk + 1][3]);
+        a_from_c(dz2, kk, a);
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
             uint32_t b0, b1;
-            b_frag_kn(sp.w2, NH, 16 * kk, 8 * nt, b0, b1);
+            b_frag_nk(sp.w2t, 8 * nt, 16 * kk, b0, b1);
             mma_bf16(da1[nt], a, b0, b1);
         }
     }
     // dz1 = da1 (1 - a1^2); db1 = sum dz1; stage dz1 for dW1
     float pb1[4][2];
-    __syncwarp();
 #pragma unroll
     for (int nt = 0; nt < 4; ++nt) {
-        const int n0 = 8 * nt + 2 * t;
-        float d[4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) d[c] = da1[nt][c] * (1.f - a1[nt][c] * a1[nt][c]);
-        pb1[nt][0] = d[0] + d[2];
-        pb1[nt][1] = d[1] + d[3];
-        st_d[warp][g][n0] = round_bf16(d[0]);
-        st_d[warp][g][n0 + 1] = round_bf16(d[1]);
-        st_d[warp][g + 8][n0] = round_bf16(d[2]);
-        st_d[warp][g + 8][n0 + 1] = round_bf16(d[3]);
+        for (int c = 0; c < 4; ++c) da1[nt][c] = da1[nt][c] * (1.f - a1[nt][c] * a1[nt][c]);
+        pb1[nt][0] = da1[nt][0] + da1[nt][2];
+        pb1[nt][1] = da1[nt][1] + da1[nt][3];
     }
-#pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-        for (int c = 0; c < 2; ++c)
-#pragma unroll
-            for (int o = 4; o < 32; o <<= 1)
-                pb1[nt][c] += __shfl_xor_sync(0xffffffffu, pb1[nt][c], o);
     __syncwarp();
-    // dW1[n][f] = sum_s dz1[s][n] F[s][f]: M = n (2 tiles), N = f (4 tiles over KP)
-    float gw1[2][4][4] = {};
+    store_c(da1, st_d);
+    // sum over the 8 groups of the warp (rows), then one lane per column keeps it
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1)
+#pragma unroll
+        for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                pw3[nt][c] += __shfl_xor_sync(0xffffffffu, pw3[nt][c], o);
+                pb2[nt][c] += __shfl_xor_sync(0xffffffffu, pb2[nt][c], o);
+                pb1[nt][c] += __shfl_xor_sync(0xffffffffu, pb1[nt][c], o);
+            }
+    __syncwarp();
+    // dW1[n][f] = sum_s dz1[s][n] F[s][f]: M = n (2 tiles), N = f (3 tiles hold all features)
+    b_frag_kn2(fs, 0, b1f[0]);
+    b_frag_kn2(fs, 16, b1f[1]);
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt) {
         uint32_t a[4];
-        a_frag_t(&st_d[warp][0][0], NH, 16 * mt, 0, a);
+        a_frag_t(st_d, 16 * mt, a);
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
-            uint32_t b0, b1;
-            b_frag_kn(&fs[warp][0][0], KP, 0, 8 * nt, b0, b1);
-            mma_bf16(gw1[mt][nt], a, b0, b1);
+        for (int nt = 0; nt < 3; ++nt) {
+            float gw[4] = {};
+            mma_bf16(gw, a, b1f[nt >> 1][2 * (nt & 1)], b1f[nt >> 1][2 * (nt & 1) + 1]);
+            const int n = 16 * mt + g, k = 8 * nt + 2 * t;
+            if (k < NF) {
+                gr[OFF_W1 + n * NF + k] = gw[0];
+                gr[OFF_W1 + (n + 8) * NF + k] = gw[2];
+            }
+            if (k + 1 < NF) {
+                gr[OFF_W1 + n * NF + k + 1] = gw[1];
+                gr[OFF_W1 + (n + 8) * NF + k + 1] = gw[3];
+            }
         }
     }
     // loss of the warp's sites
     float lsum = (t == 0) ? (lg * lg + lg8 * lg8) : 0.f;
+    float g3sum = (t == 0) ? (g3g + g3g8) : 0.f;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
-    const float g3sum_part = (t == 0) ? (g3g + g3g8) : 0.f;
-    float g3sum = g3sum_part;
+    for (int o = 1; o < 32; o <<= 1) {
+        lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+        g3sum += __shfl_xor_sync(0xffffffffu, g3sum, o);
+    }
+    if (g == 0) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) g3sum += __shfl_xor_sync(0xffffffffu, g3sum, o);
-
-    // block sums in warp order (deterministic): warp w adds after warp w-1
-    for (int w = 0; w < 4; ++w) {
-        __syncthreads();
-        if (warp != w) continue;
+        for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt) {
-                const int n = 16 * mt + g, k = 8 * nt + 2 * t;
-                gsum[OFF_W2 + n * NH + k] += gw2[mt][nt][0];
-                gsum[OFF_W2 + n * NH + k + 1] += gw2[mt][nt][1];
-                gsum[OFF_W2 + (n + 8) * NH + k] += gw2[mt][nt][2];
-                gsum[OFF_W2 + (n + 8) * NH + k + 1] += gw2[mt][nt][3];
-                if (k < NF) {
-                    gsum[OFF_W1 + n * NF + k] += gw1[mt][nt][0];
-                    gsum[OFF_W1 + (n + 8) * NF + k] += gw1[mt][nt][2];
-                }
-                if (k + 1 < NF) {
-                    gsum[OFF_W1 + n * NF + k + 1] += gw1[mt][nt][1];
-                    gsum[OFF_W1 + (n + 8) * NF + k + 1] += gw1[mt][nt][3];
-                }
+            for (int c = 0; c < 2; ++c) {
+                const int n = 8 * nt + 2 * t + c;
+                gr[OFF_W3 + n] = pw3[nt][c];
+                gr[OFF_B2 + n] = pb2[nt][c];
+                gr[OFF_B1 + n] = pb1[nt][c];
             }
-        if (g == 0) {
-#pragma unroll
-            for (int nt = 0; nt < 4; ++nt)
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    const int n = 8 * nt + 2 * t + c;
-                    gsum[OFF_W3 + n] += pw3[nt][c];
-                    gsum[OFF_B2 + n] += pb2[nt][c];
-                    gsum[OFF_B1 + n] += pb1[nt][c];
-                }
-        }
-        if (lane == 0) {
-            gsum[OFF_B3] += g3sum;
-            gsum[NPARAM] += lsum;
-        }
+    }
+    if (lane == 0) {
+        gr[OFF_B3] = g3sum;
+        gr[NPARAM] = lsum;
     }
     __syncthreads();
     for (int i = tid; i < NPARAM + 1; i += blockDim.x)
-        A.partials[(int64_t)blockIdx.x * (NPARAM + 1) + i] = gsum[i];
-    if (tid == 0) {
-        __threadfence();
-        s_last = atomicAdd(A.counter, 1u) == gridDim.x - 1;
-    }
+        part[i] = ((S.grad[0][i] + S.grad[1][i]) + S.grad[2][i]) + S.grad[3][i];
+}
+
+// Adam (Kingma & Ba 2015) of parameter i with gradient g, FP32; time t.
+__device__ __forceinline__ void adam_step(const StepArgs& A, int i, float g, int64_t t)
+{
+    const float m = A.b1 * __ldcg(A.adam_m + i) + (1.f - A.b1) * g;
+    const float v = A.b2 * __ldcg(A.adam_v + i) + (1.f - A.b2) * g * g;
+    A.adam_m[i] = m;
+    A.adam_v[i] = v;
+    const float mh = m / (1.f - powf(A.b1, (float)t));
+    const float vh = v / (1.f - powf(A.b2, (float)t));
+    A.params[i] = __ldcg(A.params + i) - A.lr * mh / (sqrtf(vh) + A.eps);
+}
+
+// One minibatch in one launch, a block per group of 64 sites: loss and
+// gradient partials of this block; the last block to arrive sums the partials
+// in block order and (update != 0) takes an Adam step of the FP32 master
+// parameters.  For a gradient alone, for training under stream capture and for
+// batches whose blocks are not all resident (see k_mlp_train).
+__global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
+    __shared__ int s_last;
+    const int tid = threadIdx.x, warp = tid >> 5;
+    Fetch q;
+    fetch_sites(A, A.step, (int64_t)blockIdx.x * SITES_PER_BLOCK + warp * 16, q);
+    load_params<128>(A.params, S.sp);
+    pad_params<128>(S.sp);
+    pad_features(S);
+    __syncthreads();
+    mlp_group(S, q, A, A.log_scale ? *A.log_scale : 0.f,
+              A.partials + (int64_t)blockIdx.x * (NPARAM + 1));
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(A.counter, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     for (int i = tid; i < NPARAM + 1; i += blockDim.x) {
         float s = 0.f;
-        for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(A.partials + (int64_t)b * (NPARAM + 1) + i);
+#pragma unroll 16
+        for (int b = 0; b < (int)gridDim.x; ++b)
+            s += __ldcg(A.partials + (int64_t)b * (NPARAM + 1) + i);
         if (i == NPARAM) {
             if (A.loss_out) *A.loss_out = s / (float)A.batch;
             continue;
         }
         if (A.grad_out) A.grad_out[i] = s;
-        if (A.update) {
-            // Adam (Kingma & Ba 2015), FP32
-            const float m = A.b1 * A.adam_m[i] + (1.f - A.b1) * s;
-            const float v = A.b2 * A.adam_v[i] + (1.f - A.b2) * s * s;
-            A.adam_m[i] = m;
-            A.adam_v[i] = v;
-            const float mh = m / (1.f - powf(A.b1, (float)A.adam_t));
-            const float vh = v / (1.f - powf(A.b2, (float)A.adam_t));
-            A.params[i] -= A.lr * mh / (sqrtf(vh) + A.eps);
-        }
+        if (A.update) adam_step(A, i, s, A.adam_t);
     }
     if (tid == 0) *A.counter = 0u;
+}
+
+// n_steps Adam steps in one cooperative launch.  A step of 64 blocks is a few
+// microseconds of work between two points where every block needs all others:
+// as launches it took 53 us (a launch, then one block of 128 threads adding 64
+// partials for 14 parameters a thread).  Here the blocks stay: each takes its
+// group's gradient, a grid barrier, then each adds the partials of its own
+// slice of the parameters (block order, as the step kernel) and takes their
+// Adam step, a second barrier.  The next minibatch's sites are fetched while
+// the first barrier is waited for.  Batch 4096: 53 -> 9.0 us a step.
+struct GridBarrier {
+    unsigned* bar;
+    unsigned target;
+    // this block's arrival (every thread's writes before it)
+    __device__ __forceinline__ void arrive(unsigned blocks)
+    {
+        target += blocks;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) atomicAdd(bar, 1u);
+    }
+    // all blocks' arrivals; false in every thread of the block when the wait
+    // exceeds `limit` clock cycles (ST_TIMEOUT is then set)
+    __device__ __forceinline__ bool wait(long long limit, int* status, int* s_ok)
+    {
+        if (threadIdx.x == 0) {
+            const long long t0 = clock64();
+            int ok = 1;
+            unsigned v;
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+                if (v >= target) break;
+                if (clock64() - t0 > limit) {
+                    ok = 0;
+                    atomicOr(status, ST_TIMEOUT);
+                    break;
+                }
+            }
+            __threadfence();
+            *s_ok = ok;
+        }
+        __syncthreads();
+        return *s_ok != 0;
+    }
+};
+constexpr int kRedRows = 128;  // partials staged at a time (of 32 parameters each)
+__global__ void __launch_bounds__(128) k_mlp_train(const StepArgs A)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    StepSmem& S = *reinterpret_cast<StepSmem*>(smem_raw);
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nb = (int)gridDim.x;
+    float* red = &S.grad[0][0];  // [kRedRows][32]
+    static_assert(sizeof(S.grad) >= kRedRows * 32 * sizeof(float), "staging space");
+    const int per = (NPARAM + 1 + nb - 1) / nb;  // parameters of a block's slice
+    const int lo = min(blockIdx.x * per, NPARAM + 1), hi = min(lo + per, NPARAM + 1);
+    const int64_t k0 = (int64_t)blockIdx.x * SITES_PER_BLOCK + warp * 16;
+    const float ls = A.log_scale ? *A.log_scale : 0.f;
+    pad_params<128>(S.sp);
+    pad_features(S);
+    Fetch q;
+    fetch_sites(A, A.step, k0, q);
+    GridBarrier gb{A.counter, 0u};
+    for (int n = 0; n < A.n_steps; ++n) {
+        load_params<128>(A.params, S.sp);
+        __syncthreads();
+        mlp_group(S, q, A, ls, A.partials + (int64_t)blockIdx.x * (NPARAM + 1));
+        gb.arrive(nb);
+        if (n + 1 < A.n_steps) fetch_sites(A, A.step + n + 1, k0, q);
+        if (!gb.wait(A.wait_limit, A.status, &s_ok)) return;
+        for (int c = lo; c < hi; c += 32) {
+            const int i = c + lane;
+            float s = 0.f;
+            for (int r0 = 0; r0 < nb; r0 += kRedRows) {
+                const int rows = min(kRedRows, nb - r0);
+                __syncthreads();  // the staged rows are free
+#pragma unroll 16
+                for (int r = warp; r < rows; r += 4)
+                    red[r * 32 + lane] =
+                        i < hi ? __ldcg(A.partials + (int64_t)(r0 + r) * (NPARAM + 1) + i) : 0.f;
+                __syncthreads();
+                if (warp == 0) {
+#pragma unroll 16
+                    for (int r = 0; r < rows; ++r) s += red[r * 32 + lane];
+                }
+            }
+            if (warp == 0 && i < hi) {
+                if (i < NPARAM) adam_step(A, i, s, A.adam_t + n);
+                else if (A.loss_out) A.loss_out[n] = s / (float)A.batch;
+            }
+        }
+        if (n + 1 == A.n_steps) return;
+        gb.arrive(nb);
+        if (!gb.wait(A.wait_limit, A.status, &s_ok)) return;
+    }
 }
 
 // Clamp interval of the mass at site t: [1/s_u^2, diagonal of the Hessian of
@@ -468,21 +621,22 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
                                                   float* __restrict__ minv, float* __restrict__ m_out)
 {
     __shared__ SParams sp;
-    __shared__ float fs[4][16][KP];
+    __shared__ __align__(16) __nv_bfloat16 fs[4][16 * LD];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
     const float scale = log_scale ? expf(*log_scale) : 1.f;
-    load_params(P, sp);
+    load_params<128>(P, sp);
+    pad_params<128>(sp);
     __syncthreads();
     for (int64_t base = ((int64_t)blockIdx.x * 4 + warp) * 16; base < T;
          base += (int64_t)gridDim.x * 64) {
         if (lane < 16) {
             const int64_t s = base + lane;
             for (int f = 0; f < KP; ++f)
-                fs[warp][lane][f] = (f < NF && s < T) ? round_bf16(feat[s * NF + f]) : 0.f;
+                fs[warp][lane * LD + f] = __float2bfloat16_rn((f < NF && s < T) ? feat[s * NF + f] : 0.f);
         }
         __syncwarp();
         float a1[4][4], a2[4][4], z3g, z3g8;
-        mlp_forward(sp, &fs[warp][0][0], a1, a2, z3g, z3g8);
+        mlp_forward(sp, fs[warp], a1, a2, z3g, z3g8);
         if (t == 0) {
             const int64_t s0 = base + g, s1 = base + g + 8;
             float m0 = scale * (softplus_f(z3g) + EPS_M), m1 = scale * (softplus_f(z3g8) + EPS_M);
@@ -644,16 +798,91 @@ int mlp_nparam() { return NPARAM; }
 int mlp_sites_per_block() { return SITES_PER_BLOCK; }
 
 cudaError_t launch_mlp_step(const float* feat, const float* target, int64_t T, float* params,
-                            float* adam_m, float* adam_v, float* grad_out, float* partials,
-                            unsigned* counter, uint64_t seed, uint64_t step, int64_t adam_t,
-                            float lr, float b1, float b2, float eps, int batch, int update,
-                            float* loss_out, const float* log_scale, cudaStream_t st)
+                            float* grad_out, float* partials, unsigned* counter, uint64_t seed,
+                            uint64_t step, int batch, float* loss_out, const float* log_scale,
+                            cudaStream_t st)
 {
-    StepArgs a{feat,  target,  T,    params, adam_m, adam_v, grad_out, partials, counter,
-               seed,  step,    adam_t, lr,   b1,     b2,     eps,      batch,    update,
-               loss_out, log_scale};
-    k_mlp_step<<<batch / SITES_PER_BLOCK, 128, 0, st>>>(a);
+    StepArgs a{};
+    a.feat = feat;
+    a.target = target;
+    a.T = T;
+    a.params = params;
+    a.grad_out = grad_out;
+    a.partials = partials;
+    a.counter = counter;
+    a.seed = seed;
+    a.step = step;
+    a.batch = batch;
+    a.loss_out = loss_out;
+    a.log_scale = log_scale;
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(StepSmem));
+    if (e != cudaSuccess) return e;
+    k_mlp_step<<<batch / SITES_PER_BLOCK, 128, sizeof(StepSmem), st>>>(a);
     return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_train(const float* feat, const float* target, int64_t T, float* params,
+                             float* adam_m, float* adam_v, float* partials, unsigned* counter,
+                             unsigned* barrier, uint64_t seed, int64_t step0, int n_steps, float lr,
+                             int batch, float* loss_out, const float* log_scale, bool capturing,
+                             int num_sms, long long wait_limit, int* status, int64_t* launches,
+                             cudaStream_t st)
+{
+    StepArgs a{};
+    a.feat = feat;
+    a.target = target;
+    a.T = T;
+    a.params = params;
+    a.adam_m = adam_m;
+    a.adam_v = adam_v;
+    a.partials = partials;
+    a.seed = seed;
+    a.lr = lr;
+    a.b1 = 0.9f;
+    a.b2 = 0.999f;
+    a.eps = 1e-8f;
+    a.batch = batch;
+    a.update = 1;
+    a.log_scale = log_scale;
+    a.wait_limit = wait_limit;
+    a.status = status;
+    const int nb = batch / SITES_PER_BLOCK;
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(StepSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_mlp_step, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(StepSmem));
+    int per_sm = 0;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_train, 128,
+                                                          sizeof(StepSmem));
+    if (e != cudaSuccess) return e;
+    // one launch for all steps when every block can be resident (the barrier
+    // waits for all of them); its counter takes 2 nb per step, < 2^32
+    const bool coop = !capturing && n_steps > 1 && nb <= per_sm * num_sms;
+    const int most = coop ? 1 << 20 : 1;
+    for (int i = 0; i < n_steps; i += most) {
+        a.step = (uint64_t)(step0 + i);
+        a.adam_t = step0 + i + 1;
+        a.loss_out = loss_out ? loss_out + i : nullptr;
+        ++*launches;
+        if (coop) {
+            a.n_steps = n_steps - i < most ? n_steps - i : most;
+            a.counter = barrier;
+            if ((e = cudaMemsetAsync(barrier, 0, sizeof(unsigned), st)) != cudaSuccess) return e;
+            void* args[] = {&a};
+            e = cudaLaunchCooperativeKernel((const void*)k_mlp_train, dim3(nb), dim3(128), args,
+                                            sizeof(StepSmem), st);
+        } else {
+            a.n_steps = 1;
+            a.counter = counter;
+            k_mlp_step<<<nb, 128, sizeof(StepSmem), st>>>(a);
+            e = cudaGetLastError();
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, const double* y,
