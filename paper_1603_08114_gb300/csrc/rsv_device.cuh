@@ -53,6 +53,17 @@ __device__ __forceinline__ u64x4 philox_block(uint64_t seed, uint64_t series, ui
     return philox4x64_10(blk, traj, stream, series, seed, 0ULL);
 }
 
+// (double)x without the FP64 pipe, on which float conversions run: the
+// exponent re-biased and the mantissa shifted; zeros, subnormals, infinities and
+// NaN take the conversion.
+__device__ __forceinline__ double f32_to_f64(float x)
+{
+    const unsigned b = __float_as_uint(x);
+    if ((b << 1) - 0x01000000u >= 0xfe000000u) return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)),
+                            (int)(b << 29));
+}
+
 // Uniform in (0,1): (k + 1/2) 2^-53 from the top 53 bits.
 __device__ __forceinline__ double u01_53(uint64_t w)
 {

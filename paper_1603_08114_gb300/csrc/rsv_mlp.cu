@@ -655,21 +655,68 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
     }
 }
 
-// Fold n snapshot rows of x ([n][T] FP32) into running (count, mean, M2).
-__global__ void k_welford(const float* __restrict__ x, int64_t n, int64_t T, int64_t count,
-                          double* __restrict__ mean, double* __restrict__ m2)
+// Fold n snapshot rows of x ([n][T] FP32) into running (count, mean, M2) by
+// Welford's recurrence, row by row.  Bound by the FP64 pipe: the recurrence's
+// seven instructions a value.  The widening of x is done on integers, and the
+// division by the row's count n_k is q = d y, q + (d - q n_k) y with y = 1/n_k
+// rounded to nearest: d - q n_k is exact (a multiple of ulp(q) below 2 n_k of
+// them), so the sum differs from d/n_k by less than 2^-51 ulp, while an FP64
+// quotient by an integer n_k lies at least 1/(2 n_k) ulp from every midpoint;
+// the result is the correctly rounded quotient for n_k < 2^48, the value a
+// division gives.  (Outside the exponents where these hold, a division.)
+// 100 rows of 2^20 sites: 2.83 -> 1.52 ms, the same bits.
+constexpr int kWelRows = 256;  // rows whose counts a block holds at a time
+__device__ __forceinline__ double div_count(double d, double n, double y)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        double m = count ? mean[t] : 0.0, s = count ? m2[t] : 0.0;
-        for (int64_t k = 0; k < n; ++k) {
-            const double v = (double)x[k * T + t];
-            const double d = v - m;
-            m += d / (double)(count + k + 1);
-            s += d * (v - m);
+    const unsigned h = (unsigned)__double2hiint(d), e = (h >> 20) & 0x7ffu;
+    if (e - 64u > 1900u)
+        return ((h << 1) | (unsigned)__double2loint(d)) == 0u ? d : d / n;
+    const double q = d * y;
+    return fma(fma(-q, n, d), y, q);
+}
+__global__ void __launch_bounds__(256) k_welford(const float* __restrict__ x, int64_t n, int64_t T,
+                                                 int64_t count, double* __restrict__ mean,
+                                                 double* __restrict__ m2)
+{
+    __shared__ double2 s_n[kWelRows];  // (n_k, 1/n_k)
+    const bool small = count + n < (int64_t(1) << 48);
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t rounds = (T + stride - 1) / stride;  // the same for every thread
+    for (int64_t i = 0; i < rounds; ++i) {
+        const int64_t t = i * stride + blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+        const bool act = t < T;
+        double m = act && count ? mean[t] : 0.0, s = act && count ? m2[t] : 0.0;
+        for (int64_t k0 = 0; k0 < n; k0 += kWelRows) {
+            const int rows = (int)(n - k0 < kWelRows ? n - k0 : kWelRows);
+            __syncthreads();
+            for (int r = threadIdx.x; r < rows; r += blockDim.x) {
+                const double nk = (double)(count + k0 + r + 1);
+                s_n[r] = make_double2(nk, 1.0 / nk);
+            }
+            __syncthreads();
+            if (!act) continue;
+            const float* xp = x + k0 * T + t;
+            auto row = [&](float xv, int r) {
+                const double v = f32_to_f64(xv);
+                const double d = v - m;
+                m += small ? div_count(d, s_n[r].x, s_n[r].y) : d / s_n[r].x;
+                s += d * (v - m);
+            };
+            constexpr int U = 8;  // rows in flight
+            int r = 0;
+            for (; r + U <= rows; r += U) {
+                float v[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) v[u] = xp[(r + u) * T];
+#pragma unroll
+                for (int u = 0; u < U; ++u) row(v[u], r + u);
+            }
+            for (; r < rows; ++r) row(xp[r * T], r);
         }
-        mean[t] = m;
-        m2[t] = s;
+        if (act) {
+            mean[t] = m;
+            m2[t] = s;
+        }
     }
 }
 
@@ -899,7 +946,8 @@ cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, c
 cudaError_t launch_welford(const float* x, int64_t n, int64_t T, int64_t count, double* mean,
                            double* m2, cudaStream_t st)
 {
-    k_welford<<<grid1(T), 256, 0, st>>>(x, n, T, count, mean, m2);
+    const int64_t g = (T + 255) / 256;
+    k_welford<<<(unsigned)(g < 65536 ? g : 65536), 256, 0, st>>>(x, n, T, count, mean, m2);
     return cudaGetLastError();
 }
 
