@@ -29,9 +29,11 @@ rsv_status rsv_welford_target(rsv_ctx* c, const double* mean, const double* m2, 
     if (st != RSV_OK) return st;
     if (!mean || !m2 || !target_out) return fail(RSV_EINVAL, "null argument");
     if (T < 1 || count < 2) return fail(RSV_EINVAL, "need T >= 1 and count >= 2");
+    // (the context's partials hold 4096 doubles from its creation on)
     cudaError_t e = counted(c, launch_welford_target, mean, m2, T, count, hbar_out, target_out,
-                            log_scale_out, (cudaStream_t)stream);
-    if (log_scale_out) ++c->launches;
+                            log_scale_out, c->partials.as<double>(),
+                            reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter + 3),
+                            (cudaStream_t)stream);
     return e == cudaSuccess ? RSV_OK : cuda_fail(e, "welford target kernel");
 }
 
@@ -46,11 +48,11 @@ rsv_status rsv_mass_features(rsv_ctx* c, const double* y, const double* lnrv, co
     if (!theta_ok(theta)) return fail(RSV_EINVAL, "invalid theta");
     const int g = feat_grid(T);
     if ((st = c->batch.ensure((size_t)(g * 20 + 32) * sizeof(double))) != RSV_OK) return st;
-    double* part = c->batch.as<double>();
-    c->launches += 4;
-    cudaError_t e = launch_features(y, lnrv, hbar, T, to_dev(theta), feat_out, stats_out, part + 32,
+    c->launches += 2;
+    cudaError_t e = launch_features(y, lnrv, hbar, T, to_dev(theta), feat_out, stats_out,
+                                    c->batch.as<double>(),
                                     reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter + 1),
-                                    part, (cudaStream_t)stream);
+                                    (cudaStream_t)stream);
     return e == cudaSuccess ? RSV_OK : cuda_fail(e, "feature kernels");
 }
 

@@ -599,20 +599,13 @@ __global__ void __launch_bounds__(128) k_mlp_train(const StepArgs A)
     }
 }
 
-// Clamp interval of the mass at site t: [1/s_u^2, diagonal of the Hessian of
-// S at hbar] = [1/s_u^2, A_t/s_eta^2 + 1/s_u^2 + (y_t^2/2) e^{-hbar_t}], A_t =
-// 1 + phi^2 inside, 1 at the ends, 1 - phi^2 when T = 1.
-__device__ __forceinline__ float clamp_mass(float m, int64_t t, int64_t T, const double* y,
-                                            const double* hbar, const ThetaD& th)
-{
-    const double A = T == 1 ? 1.0 - th.phi * th.phi
-                   : (t == 0 || t == T - 1) ? 1.0 : 1.0 + th.phi * th.phi;
-    const double lo = 1.0 / th.su2;
-    const double hi = A / th.se2 + lo + 0.5 * y[t] * y[t] * exp(-hbar[t]);
-    return fminf(fmaxf(m, (float)lo), (float)hi);
-}
-
-// m_t for every site, clamped; writes 1/m_t (and m_t if m_out).
+// m_t for every site, clamped to [1/s_u^2, diagonal of the Hessian of S at
+// hbar] = [1/s_u^2, A_t/s_eta^2 + 1/s_u^2 + (y_t^2/2) e^{-hbar_t}], A_t = 1 +
+// phi^2 inside, 1 at the ends, 1 - phi^2 when T = 1; writes 1/m_t (and m_t if
+// m_out).  A warp takes 32 sites: two tiles through the network, then one site
+// per lane for the output and its clamp, whose FP64 instructions cost the same
+// for one active lane as for 32 (taken by 8 lanes a tile they were most of the
+// kernel).  2^20 sites: 305 -> 81 us.
 __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat, int64_t T,
                                                   const float* __restrict__ P,
                                                   const double* __restrict__ y,
@@ -621,37 +614,55 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
                                                   float* __restrict__ minv, float* __restrict__ m_out)
 {
     __shared__ SParams sp;
-    __shared__ __align__(16) __nv_bfloat16 fs[4][16 * LD];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+    __shared__ __align__(16) __nv_bfloat16 fs[4][32 * LD];
+    __shared__ u64 s_exp[kExpN];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const float scale = log_scale ? expf(*log_scale) : 1.f;
     load_params<128>(P, sp);
     pad_params<128>(sp);
+    exp_table(s_exp);
+    for (int i = tid; i < 4 * 32 * (KP - NF); i += 128)
+        fs[0][(i / (KP - NF)) * LD + NF + i % (KP - NF)] = __float2bfloat16_rn(0.f);
     __syncthreads();
-    for (int64_t base = ((int64_t)blockIdx.x * 4 + warp) * 16; base < T;
-         base += (int64_t)gridDim.x * 64) {
-        if (lane < 16) {
-            const int64_t s = base + lane;
-            for (int f = 0; f < KP; ++f)
-                fs[warp][lane * LD + f] = __float2bfloat16_rn((f < NF && s < T) ? feat[s * NF + f] : 0.f);
+    const double lo = 1.0 / th.su2;
+    const double in = (1.0 + th.phi * th.phi) / th.se2 + lo;
+    const double end = (T == 1 ? 1.0 - th.phi * th.phi : 1.0) / th.se2 + lo;
+    const float lof = (float)lo;
+    for (int64_t base = ((int64_t)blockIdx.x * 4 + warp) * 32; base < T;
+         base += (int64_t)gridDim.x * 128) {
+        const int64_t s = base + lane;
+        const bool act = s < T;
+        const double yv = act ? y[s] : 0.0, hv = act ? hbar[s] : 0.0;
+        const int64_t nf = (T - base < 32 ? T - base : 32) * NF;
+        float v[NF];  // the warp's 32 x NF features with consecutive lanes
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            const int e = lane + 32 * i;
+            v[i] = e < nf ? feat[base * NF + e] : 0.f;
         }
         __syncwarp();
-        float a1[4][4], a2[4][4], z3g, z3g8;
-        mlp_forward(sp, fs[warp], a1, a2, z3g, z3g8);
-        if (t == 0) {
-            const int64_t s0 = base + g, s1 = base + g + 8;
-            float m0 = scale * (softplus_f(z3g) + EPS_M), m1 = scale * (softplus_f(z3g8) + EPS_M);
-            if (s0 < T) m0 = clamp_mass(m0, s0, T, y, hbar, th);
-            if (s1 < T) m1 = clamp_mass(m1, s1, T, y, hbar, th);
-            if (s0 < T) {
-                minv[s0] = 1.f / m0;
-                if (m_out) m_out[s0] = m0;
-            }
-            if (s1 < T) {
-                minv[s1] = 1.f / m1;
-                if (m_out) m_out[s1] = m1;
-            }
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            const int e = lane + 32 * i;
+            fs[warp][(e / NF) * LD + e % NF] = __float2bfloat16_rn(v[i]);
         }
         __syncwarp();
+        float z = 0.f;
+#pragma unroll 1
+        for (int tile = 0; tile < 2; ++tile) {
+            float a1[4][4], a2[4][4], zg, zg8;
+            mlp_forward(sp, fs[warp] + tile * 16 * LD, a1, a2, zg, zg8);
+            // lane r of the tile's 16 takes row r (held by the lanes of group r & 7)
+            const float u = __shfl_sync(0xffffffffu, zg, (lane & 7) * 4);
+            const float w = __shfl_sync(0xffffffffu, zg8, (lane & 7) * 4);
+            if ((lane >> 4) == tile) z = (lane & 8) ? w : u;
+        }
+        if (act) {
+            const double hi = (s == 0 || s == T - 1 ? end : in) + 0.5 * yv * yv * exp_neg(hv, s_exp);
+            const float m = fminf(fmaxf(scale * (softplus_f(z) + EPS_M), lof), (float)hi);
+            minv[s] = 1.f / m;
+            if (m_out) m_out[s] = m;
+        }
     }
 }
 
@@ -720,115 +731,203 @@ __global__ void __launch_bounds__(256) k_welford(const float* __restrict__ x, in
     }
 }
 
-// target_t = log(1 / Var(h_t)) = log((count - 1) / M2_t); hbar_t = mean_t.
-__global__ void k_welford_target(const double* __restrict__ mean, const double* __restrict__ m2,
-                                 int64_t T, int64_t count, double* __restrict__ hbar,
-                                 float* __restrict__ target)
+// Sums of one value per block, for a last-block finish: true in every thread
+// of the last block to arrive.
+__device__ __forceinline__ bool last_block(unsigned* counter, int* s_last)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        if (hbar) hbar[t] = mean[t];
-        const double var = m2[t] / (double)(count - 1);
-        target[t] = (float)log(1.0 / fmax(var, 1e-300));
-    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) *s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!*s_last) return false;
+    __threadfence();
+    if (threadIdx.x == 0) *counter = 0u;
+    return true;
 }
 
-// log s = mean over the sites of the target (one block, FP64, fixed order).
-__global__ void __launch_bounds__(1024) k_target_mean(const float* __restrict__ target, int64_t T,
-                                                      float* __restrict__ out)
-{
-    __shared__ double red[32];
-    double s = 0.0;
-    for (int64_t t = threadIdx.x; t < T; t += blockDim.x) s += (double)target[t];
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) *out = (float)(s / (double)T);
-}
-
-// Raw features of each site (see the header of oracle/mlp.py for the list).
-__global__ void k_feat_raw(const double* __restrict__ y, const double* __restrict__ lnrv,
-                           const double* __restrict__ hbar, int64_t T, ThetaD th,
-                           float* __restrict__ F)
-{
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        float* f = F + t * NF;
-        const double yt = y[t];
-        f[0] = (float)(yt * yt);
-        f[1] = (float)lnrv[t];
-        for (int k = -4; k <= 4; ++k) {
-            const int64_t s = t + k;
-            f[2 + k + 4] = (s >= 0 && s < T) ? (float)hbar[s] : 0.f;
-        }
-        f[11] = (float)th.phi;
-        f[12] = (float)th.mu;
-        f[13] = (float)th.xi;
-        f[14] = (float)th.se2;
-        f[15] = (float)th.su2;
-        const int64_t d = t < T - 1 - t ? t : T - 1 - t;   // distance to the nearer end
-        f[16] = ldexpf(1.f, -(int)(d < 64 ? d : 64));
-        f[17] = (float)((1.0 + th.phi * th.phi) / th.se2);
-        f[18] = (float)(1.0 / th.su2);
-        f[19] = (float)(0.5 * yt * yt * exp(-hbar[t]));
-    }
-}
-
-// Column sums (pass 0: sum f; pass 1: sum (f - mean)^2) with a last-block
-// finish; stats = [mean(20), inv_sd(20)].
-__global__ void __launch_bounds__(256) k_feat_stats(const float* __restrict__ F, int64_t T,
-                                                    int pass, double* __restrict__ partials,
-                                                    unsigned* __restrict__ counter,
-                                                    double* __restrict__ acc,
-                                                    float* __restrict__ stats)
+// target_t = log(1 / Var(h_t)) = log((count - 1) / M2_t); hbar_t = mean_t; and
+// log s = the mean over the sites of the target (FP64, fixed order), if asked
+// for (one block over all sites took 0.59 ms for it at 2^20 sites).
+__global__ void __launch_bounds__(256) k_welford_target(
+    const double* __restrict__ mean, const double* __restrict__ m2, int64_t T, int64_t count,
+    double* __restrict__ hbar, float* __restrict__ target, float* __restrict__ log_scale,
+    double* __restrict__ partials, unsigned* __restrict__ counter)
 {
     __shared__ double red[32];
     __shared__ int s_last;
-    double loc[NF];
-    for (int f = 0; f < NF; ++f) loc[f] = 0.0;
+    const double nk = (double)(count - 1), inv = 1.0 / nk;
+    const bool small = count < (int64_t(1) << 48);
+    double sum = 0.0;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
-         t += (int64_t)gridDim.x * blockDim.x)
-        for (int f = 0; f < NF; ++f) {
-            const double v = (double)F[t * NF + f];
-            if (pass == 0) {
-                loc[f] += v;
-            } else {
-                const double d = v - acc[f];
-                loc[f] += d * d;
-            }
-        }
-    for (int f = 0; f < NF; ++f) {
-        const double b = block_sum(loc[f], red);
-        if (threadIdx.x == 0) partials[(int64_t)blockIdx.x * NF + f] = b;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        if (hbar) hbar[t] = mean[t];
+        const double var = small ? div_count(m2[t], nk, inv) : m2[t] / nk;
+        const float v = (float)log(1.0 / fmax(var, 1e-300));
+        target[t] = v;
+        if (log_scale) sum += f32_to_f64(v);
     }
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (threadIdx.x < NF) {
-        const int f = threadIdx.x;
-        double s = 0.0;
-        for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(partials + (int64_t)b * NF + f);
-        if (pass == 0) {
-            acc[f] = s / (double)T;
-            stats[f] = f == EDGE ? 0.f : (float)acc[f];
-        } else {
-            const double sd = sqrt(s / (double)T);
-            const double m = acc[f];
-            stats[NF + f] = f == EDGE ? 1.f
-                          : (sd > 1e-12 * fmax(1.0, fabs(m))) ? (float)(1.0 / sd) : 0.f;
-        }
-    }
-    if (threadIdx.x == 0) *counter = 0u;
+    if (!log_scale) return;
+    sum = block_sum(sum, red);
+    if (threadIdx.x == 0) partials[blockIdx.x] = sum;
+    if (!last_block(counter, &s_last)) return;
+    sum = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) sum += __ldcg(partials + i);
+    sum = block_sum(sum, red);
+    if (threadIdx.x == 0) *log_scale = (float)(sum / (double)T);
 }
 
-__global__ void k_feat_norm(float* __restrict__ F, int64_t T, const float* __restrict__ stats)
+// The raw features of a site that depend on it (FP32): y^2, lnRV, hbar and
+// (y^2/2) e^{-hbar}.  The other features are hbar of the eight sites around it
+// (0 past the ends), constants of theta, and the edge proximity.
+struct SiteFeat {
+    float y2, lr, hb, ey;
+};
+__device__ __forceinline__ SiteFeat site_features(double y, double lr, double hb, const u64* s_exp)
 {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < T * NF;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int f = (int)(i % NF);
-        F[i] = fminf(fmaxf((F[i] - stats[f]) * stats[NF + f], -CLIP), CLIP);
+    return SiteFeat{(float)(y * y), (float)lr, (float)hb, (float)(0.5 * y * y * exp_neg(hb, s_exp))};
+}
+__device__ __forceinline__ float const_feature(int f, const ThetaD& th)
+{
+    switch (f) {
+        case 11: return (float)th.phi;
+        case 12: return (float)th.mu;
+        case 13: return (float)th.xi;
+        case 14: return (float)th.se2;
+        case 15: return (float)th.su2;
+        case 17: return (float)((1.0 + th.phi * th.phi) / th.se2);
+        default: return (float)(1.0 / th.su2);  // 18
+    }
+}
+
+// Mean and 1/sd of every feature over the sites, stats = [mean(20), inv_sd(20)]:
+// one pass over the inputs (24 B a site), sums in FP64 of the four site
+// features about their values at the middle site; the nine hbar columns are
+// the same values up to the few at the ends, constants are exact.  (The
+// features were written out, 80 B a site, read back twice for the statistics
+// and once to be standardised in place: 640 us at 2^20 sites, 110 now.)
+constexpr int kFeatSums = 8;
+__global__ void __launch_bounds__(256) k_feat_stats(const double* __restrict__ y,
+                                                    const double* __restrict__ lnrv,
+                                                    const double* __restrict__ hbar, int64_t T,
+                                                    ThetaD th, double* __restrict__ partials,
+                                                    unsigned* __restrict__ counter,
+                                                    float* __restrict__ stats)
+{
+    __shared__ double red[32], tot[kFeatSums];
+    __shared__ u64 s_exp[kExpN];
+    __shared__ int s_last;
+    exp_table(s_exp);
+    __syncthreads();
+    const int64_t mid = T / 2;
+    const SiteFeat c = site_features(y[mid], lnrv[mid], hbar[mid], s_exp);
+    const float cv[4] = {c.y2, c.lr, c.hb, c.ey};
+    double cf[4];  // the centres (any finite value serves)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) cf[i] = isfinite(cv[i]) ? (double)cv[i] : 0.0;
+    double sum[kFeatSums];
+#pragma unroll
+    for (int i = 0; i < kFeatSums; ++i) sum[i] = 0.0;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const SiteFeat q = site_features(y[t], lnrv[t], hbar[t], s_exp);
+        const float v[4] = {q.y2, q.lr, q.hb, q.ey};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double d = f32_to_f64(v[i]) - cf[i];
+            sum[2 * i] += d;
+            sum[2 * i + 1] = fma(d, d, sum[2 * i + 1]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < kFeatSums; ++i) {
+        const double b = block_sum(sum[i], red);
+        if (threadIdx.x == 0) partials[(int64_t)blockIdx.x * kFeatSums + i] = b;
+    }
+    if (!last_block(counter, &s_last)) return;
+    {   // warp i adds sum i over the blocks
+        const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        static_assert(kFeatSums * 32 == 256, "one warp per sum");
+        double v = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32)
+            v += __ldcg(partials + (int64_t)b * kFeatSums + i);
+        v = warp_sum(v);
+        if (lane == 0) tot[i] = v;
+    }
+    __syncthreads();
+    const int f = threadIdx.x;
+    if (f >= NF) return;
+    double s1 = 0.0, s2 = 0.0, cen = 0.0;
+    if (f == 0 || f == 1 || f == 19) {
+        const int i = f == 19 ? 3 : f;
+        cen = cf[i];
+        s1 = tot[2 * i];
+        s2 = tot[2 * i + 1];
+    } else if (f >= 2 && f <= 10) {
+        // column of hbar_{t+k}: the values without the first k (last -k) ones, and as many zeros
+        const int k = f - 6, n = (int)(T < (k < 0 ? -k : k) ? T : (k < 0 ? -k : k));
+        cen = cf[2];
+        s1 = tot[4];
+        s2 = tot[5];
+        for (int j = 0; j < n; ++j) {
+            const double d = (double)(float)hbar[k > 0 ? j : T - 1 - j] - cen;
+            s1 -= d + cen;
+            s2 += cen * cen - d * d;
+        }
+    } else if (f != EDGE) {
+        cen = (double)const_feature(f, th);
+    }
+    const double dm = s1 / (double)T, m = cen + dm;
+    const double sd = sqrt(fmax(s2 / (double)T - dm * dm, 0.0));
+    stats[f] = f == EDGE ? 0.f : (float)m;
+    stats[NF + f] = f == EDGE ? 1.f : (sd > 1e-12 * fmax(1.0, fabs(m))) ? (float)(1.0 / sd) : 0.f;
+}
+
+// The standardised, clipped features, 256 sites a block, staged in shared
+// memory and written with consecutive lanes.
+__global__ void __launch_bounds__(256) k_feat_write(const double* __restrict__ y,
+                                                    const double* __restrict__ lnrv,
+                                                    const double* __restrict__ hbar, int64_t T,
+                                                    ThetaD th, const float* __restrict__ stats,
+                                                    float* __restrict__ F)
+{
+    __shared__ float s_f[256 * NF], s_hb[256 + 8], s_m[NF], s_i[NF], s_c[NF];
+    __shared__ u64 s_exp[kExpN];
+    const int tid = threadIdx.x;
+    exp_table(s_exp);
+    if (tid < NF) {
+        s_m[tid] = stats[tid];
+        s_i[tid] = stats[NF + tid];
+        s_c[tid] = const_feature(tid, th);
+    }
+    for (int64_t t0 = (int64_t)blockIdx.x * 256; t0 < T; t0 += (int64_t)gridDim.x * 256) {
+        __syncthreads();
+        const int64_t t = t0 + tid;
+        const bool act = t < T;
+        const SiteFeat q = site_features(act ? y[t] : 0.0, act ? lnrv[t] : 0.0, act ? hbar[t] : 0.0,
+                                         s_exp);
+        s_hb[tid + 4] = act ? q.hb : 0.f;
+        if (tid < 8) {
+            const int64_t s = tid < 4 ? t0 - 4 + tid : t0 + 256 + (tid - 4);
+            s_hb[tid < 4 ? tid : 256 + tid] = (s >= 0 && s < T) ? (float)hbar[s] : 0.f;
+        }
+        __syncthreads();
+        auto put = [&](int f, float v) {
+            s_f[tid * NF + f] = fminf(fmaxf((v - s_m[f]) * s_i[f], -CLIP), CLIP);
+        };
+        const int64_t d = t < T - 1 - t ? t : T - 1 - t;  // distance to the nearer end
+        put(0, q.y2);
+        put(1, q.lr);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) put(2 + k, s_hb[tid + k]);
+#pragma unroll
+        for (int f = 11; f < 16; ++f) put(f, s_c[f]);
+        put(16, ldexpf(1.f, -(int)(d < 64 ? d : 64)));
+        put(17, s_c[17]);
+        put(18, s_c[18]);
+        put(19, q.ey);
+        __syncthreads();
+        const int n = (int)(T - t0 < 256 ? T - t0 : 256) * NF;
+        for (int i = tid; i < n; i += 256) F[t0 * NF + i] = s_f[i];
     }
 }
 
@@ -936,8 +1035,8 @@ cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, c
                             const double* hbar, ThetaD th, const float* log_scale, float* minv,
                             float* m_out, cudaStream_t st)
 {
-    int64_t g = (T + 63) / 64;
-    if (g > 152 * 16) g = 152 * 16;
+    int64_t g = (T + 127) / 128;
+    if (g > 152 * 8) g = 152 * 8;
     k_mlp_mass<<<(int)(g < 1 ? 1 : g), 128, 0, st>>>(feat, T, params, y, hbar, th, log_scale,
                                                       minv, m_out);
     return cudaGetLastError();
@@ -952,10 +1051,11 @@ cudaError_t launch_welford(const float* x, int64_t n, int64_t T, int64_t count, 
 }
 
 cudaError_t launch_welford_target(const double* mean, const double* m2, int64_t T, int64_t count,
-                                  double* hbar, float* target, float* log_scale, cudaStream_t st)
+                                  double* hbar, float* target, float* log_scale, double* partials,
+                                  unsigned* counter, cudaStream_t st)
 {
-    k_welford_target<<<grid1(T), 256, 0, st>>>(mean, m2, T, count, hbar, target);
-    if (log_scale) k_target_mean<<<1, 1024, 0, st>>>(target, T, log_scale);
+    k_welford_target<<<grid1(T), 256, 0, st>>>(mean, m2, T, count, hbar, target, log_scale,
+                                               partials, counter);
     return cudaGetLastError();
 }
 
@@ -963,13 +1063,12 @@ int feat_grid(int64_t T) { return grid1(T); }
 
 cudaError_t launch_features(const double* y, const double* lnrv, const double* hbar, int64_t T,
                             ThetaD th, float* F, float* stats, double* partials, unsigned* counter,
-                            double* acc, cudaStream_t st)
+                            cudaStream_t st)
 {
+    // two blocks per SM: a block's FP64 reductions cost as much as a few hundred sites
     const int g = grid1(T);
-    k_feat_raw<<<g, 256, 0, st>>>(y, lnrv, hbar, T, th, F);
-    k_feat_stats<<<g, 256, 0, st>>>(F, T, 0, partials, counter, acc, stats);
-    k_feat_stats<<<g, 256, 0, st>>>(F, T, 1, partials, counter, acc, stats);
-    k_feat_norm<<<grid1(T * NF), 256, 0, st>>>(F, T, stats);
+    k_feat_stats<<<g < 304 ? g : 304, 256, 0, st>>>(y, lnrv, hbar, T, th, partials, counter, stats);
+    k_feat_write<<<g, 256, 0, st>>>(y, lnrv, hbar, T, th, stats, F);
     return cudaGetLastError();
 }
 
