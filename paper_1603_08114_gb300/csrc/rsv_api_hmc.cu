@@ -252,24 +252,17 @@ rsv_status run(rsv_ctx* c, const Plan& P, const RunOpts& o, cudaStream_t s)
         if ((e = counted(c, launch_theta_prep, o.theta, o.th_inline, (int)n, c->rho,
                          c->theta_f.as<MixedTheta>(), s)) != cudaSuccess)
             return cuda_fail(e, "theta prep kernel");
-        if ((e = counted(c, launch_prep_mixed, o.y, o.lnrv, c->a_f.as<float>(),
-                         c->lr_f.as<float2>(), P.total, s)) != cudaSuccess)
-            return cuda_fail(e, "prep kernel");
-        if ((e = counted(c, launch_h_to_ff, (const double*)o.h, c->fbuf0.as<float2>(), P.total,
-                         s)) != cudaSuccess)
-            return cuda_fail(e, "state split kernel");
         // without leverage dH takes the start's potential energy from the
         // statistics of the state; the kernel keeps them for both buffers
         a.rstats = c->rstats.as<StatsRec>();
-        if (!P.lev) {
-            c->launches += 1;  // two kernels
-            if ((e = counted(c, launch_state_stats, P, (const float2*)c->fbuf0.as<float2>(),
-                             (const float*)c->a_f.as<float>(),
-                             (const float2*)c->lr_f.as<float2>(),
-                             (const MixedTheta*)c->theta_f.as<MixedTheta>(),
-                             c->partials.as<double>(), c->rstats.as<StatsRec>(), s)) != cudaSuccess)
-                return cuda_fail(e, "state statistics kernels");
-        }
+        e = P.lev ? counted(c, launch_prep_mixed, (const double*)o.h, o.y, o.lnrv,
+                            c->fbuf0.as<float2>(), c->a_f.as<float>(), c->lr_f.as<float2>(), P.total, s)
+                  : counted(c, launch_prep_stats, P, (const double*)o.h, o.y, o.lnrv,
+                            c->fbuf0.as<float2>(), c->a_f.as<float>(), c->lr_f.as<float2>(),
+                            (const MixedTheta*)c->theta_f.as<MixedTheta>(),
+                            c->partials.as<double>(), c->ser_cnt.as<unsigned>(),
+                            c->rstats.as<StatsRec>(), s);
+        if (e != cudaSuccess) return cuda_fail(e, "prep kernel");
     } else {
         a.h0d = o.h;
         a.h1d = c->dbuf0.as<double>();

@@ -55,11 +55,13 @@ __device__ __forceinline__ u64x4 philox_block(uint64_t seed, uint64_t series, ui
 
 // (double)x without the FP64 pipe, on which float conversions run: the
 // exponent re-biased and the mantissa shifted; zeros, subnormals, infinities and
-// NaN take the conversion.
+// NaN take the conversion, out of line: inlined it would be predicated into
+// every warp, and a predicated FP64 instruction occupies the pipe all the same.
+static __device__ __noinline__ double f32_to_f64_slow(float x) { return (double)x; }
 __device__ __forceinline__ double f32_to_f64(float x)
 {
     const unsigned b = __float_as_uint(x);
-    if ((b << 1) - 0x01000000u >= 0xfe000000u) return (double)x;
+    if ((b << 1) - 0x01000000u >= 0xfe000000u) return f32_to_f64_slow(x);
     return __hiloint2double((int)((b & 0x80000000u) | (((b >> 3) & 0x0fffffffu) + 0x38000000u)),
                             (int)(b << 29));
 }
@@ -157,6 +159,37 @@ __host__ __device__ __forceinline__ ff ff_from_double(double d)
     return {h, (float)(d - (double)h)};
 }
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }
+// (float)d for kernels over many sites: the rounding to nearest even on the
+// integer units (conversions run on the FP64 pipe, 2 lanes per cycle and SM).
+// 2^-73 <= |d| < 2^127; others convert (out of line, see f32_to_f64).
+static __device__ __noinline__ float f64_to_f32_slow(double d) { return (float)d; }
+static __device__ __noinline__ ff ff_split_slow(double d) { return ff_from_double(d); }
+__device__ __forceinline__ float f64_to_f32(double d)
+{
+    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+    const unsigned E = (h >> 20) & 0x7ffu;
+    if (E - 950u > 199u) return f64_to_f32_slow(d);
+    unsigned fb = __funnelshift_l(l, h, 3) - 0xc0000000u;  // exponent re-biased, top 23 mantissa bits
+    fb += ((l & 0x1fffffffu) + 0x0fffffffu + (fb & 1u)) >> 29;
+    return __uint_as_float(fb | (h & 0x80000000u));
+}
+// ff_from_double likewise, the same bits: the 29 mantissa bits below the float
+// (signed, after its rounding) become the small part, exactly converted in two
+// pieces and rounded once.
+__device__ __forceinline__ ff ff_split(double d)
+{
+    const unsigned h = (unsigned)__double2hiint(d), l = (unsigned)__double2loint(d);
+    const unsigned E = (h >> 20) & 0x7ffu, sign = h & 0x80000000u;
+    if (E - 950u > 199u) return ff_split_slow(d);
+    unsigned fb = __funnelshift_l(l, h, 3) - 0xc0000000u;
+    const unsigned r = l & 0x1fffffffu, up = (r + 0x0fffffffu + (fb & 1u)) >> 29;
+    fb += up;
+    const int D = (int)r - (int)(up << 29);  // |D| <= 2^28, in units of 2^(E - 1075)
+    const float Dh = __fsub_rn(__uint_as_float((unsigned)(0x4b400000 + (D >> 8))), 12582912.0f);
+    const float Dl = __fsub_rn(__uint_as_float(0x4b000000u | (unsigned)(D & 0xff)), 8388608.0f);
+    const float m = __fmul_rn(__fmaf_rn(Dh, 256.0f, Dl), __uint_as_float((E - 948u) << 23));
+    return {__uint_as_float(fb | sign), __fadd_rn(__uint_as_float(__float_as_uint(m) ^ sign), 0.0f)};
+}
 
 // Table of 2^(j/32), j = 0..31, as double-float pairs (filled by ff_exp_table).
 __device__ __forceinline__ void ff_exp_table(float2* tab)

@@ -270,15 +270,32 @@ __global__ void k_commit_fp64(double* __restrict__ h, const double* __restrict__
     }
 }
 
-__global__ void k_prep_mixed(const double* __restrict__ y, const double* __restrict__ lnrv,
+// y^2/2 as FP32 with the sign of y (for the leverage term): the square on the
+// FP64 pipe, its half and rounding on the integer units (the bits of
+// (float)(0.5 y y)).
+static __device__ __noinline__ float half_square_slow(double y) { return (float)(0.5 * y * y); }
+__device__ __forceinline__ float signed_half_square(double y)
+{
+    const double q = y * y;
+    const unsigned h = (unsigned)__double2hiint(q);
+    const float a = ((h >> 20) & 0x7ffu) - 951u > 198u
+                        ? half_square_slow(y)
+                        : f64_to_f32(__hiloint2double((int)(h - 0x00100000u), __double2loint(q)));
+    return __uint_as_float(__float_as_uint(a) | ((unsigned)__double2hiint(y) & 0x80000000u));
+}
+
+// Per-site constants and the state as (hi, lo) pairs, elementwise (the leverage
+// model; without leverage k_prep_stats does both and the state's statistics).
+__global__ void k_prep_mixed(const double* __restrict__ h, const double* __restrict__ y,
+                             const double* __restrict__ lnrv, float2* __restrict__ hf,
                              float* __restrict__ a_f, float2* __restrict__ lr_f, int64_t T)
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const double a = 0.5 * y[t] * y[t];
-        a_f[t] = copysignf((float)a, (float)y[t]);  // the sign of y for the leverage term
-        const ff l = ff_from_double(lnrv[t]);
+        a_f[t] = signed_half_square(y[t]);
+        const ff l = ff_split(lnrv[t]), v = ff_split(h[t]);
         lr_f[t] = make_float2(l.hi, l.lo);
+        hf[t] = make_float2(v.hi, v.lo);
     }
 }
 
@@ -286,7 +303,7 @@ __global__ void k_h_to_ff(const double* __restrict__ h, float2* __restrict__ hf,
 {
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
          t += (int64_t)gridDim.x * blockDim.x) {
-        const ff v = ff_from_double(h[t]);
+        const ff v = ff_split(h[t]);
         hf[t] = make_float2(v.hi, v.lo);
     }
 }
@@ -303,38 +320,59 @@ __device__ __forceinline__ int series_of(const SerInfo* ser, int n, int64_t t)
     return lo;
 }
 
-__global__ void k_finalize(const SerInfo* __restrict__ ser, int n, int64_t total,
-                           const int* __restrict__ cur, const int* __restrict__ acc,
-                           const double* __restrict__ h1d, const float2* __restrict__ h0f,
-                           const float2* __restrict__ h1f, double* __restrict__ h)
+// The current state back into h: run blockIdx.x of `run` sites of a single
+// series (segs NULL), or the owned sites of segment blockIdx.x, whose series it
+// knows (a search for the series of every packed site was half of the 161 us
+// for 17.7 M sites of 4096 series; the other half FP64 conversions, now one
+// FP64 addition a site: 57 us).
+__global__ void __launch_bounds__(256) k_finalize(
+    const Seg* __restrict__ segs, const SerInfo* __restrict__ ser, int64_t total, int run,
+    const int* __restrict__ cur, const int* __restrict__ acc, const double* __restrict__ h1d,
+    const float2* __restrict__ h0f, const float2* __restrict__ h1f, double* __restrict__ h)
 {
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int s = n > 1 ? series_of(ser, n, t) : 0;
-        const int c = cur ? cur[s] : 0;
+    int s = 0;
+    int64_t lo = (int64_t)blockIdx.x * run, hi = lo + run < total ? lo + run : total;
+    if (segs) {
+        const Seg g = segs[blockIdx.x];
+        s = g.series;
+        lo = ser[s].off + g.lo;
+        hi = ser[s].off + g.hi;
+    }
+    const int c = cur ? cur[s] : 0;
+    if (h0f ? acc && acc[s] == 0 : c == 0) return;
+    const float2* hf = c ? h1f : h0f;
+#pragma unroll 4
+    for (int64_t t = lo + threadIdx.x; t < hi; t += 256) {
         if (h0f) {
-            if (acc && acc[s] == 0) continue;
-            const float2 v = (c ? h1f : h0f)[t];
-            h[t] = (double)v.x + (double)v.y;
-        } else if (c) {
+            const float2 v = hf[t];
+            h[t] = f32_to_f64(v.x) + f32_to_f64(v.y);
+        } else {
             h[t] = h1d[t];
         }
     }
 }
 
-// The statistics (StateStats) of the state hf: one block per segment over its
-// owned sites (a thread's sites in order, then a butterfly in each warp and
-// the warps in order), written as kPartialWords double-floats per segment
-// (sum lnRV, the statistics, sum lnRV^2); then one warp per series adds its
-// tiles and files the record as buffer 0's.
+// Per-site constants, the state as (hi, lo) pairs and its statistics
+// (StateStats): one block per segment over its owned sites (a thread's sites in
+// order, then a butterfly in each warp and the warps in order); a series'
+// record, filed as buffer 0's, by the block of a whole series or by the last
+// of a split one's tiles to arrive, whose kPartialWords double-floats (sum
+// lnRV, the statistics, sum lnRV^2) lane l adds for tiles l, l + 32, ... in
+// order, then a butterfly per value.  One pass over HBM, 44 B a site, the
+// conversions on the integer units; bound by issue, about 500 instructions a
+// site, most of them the double-float sums.  17.7 M sites: 270 us (570 as four
+// kernels with FP64 conversions); 2^22: 64 us (155).
 constexpr int kStatsThreads = 512;
-__global__ void __launch_bounds__(kStatsThreads) k_state_stats(
-    const Seg* __restrict__ segs, const SerInfo* __restrict__ ser, const float2* __restrict__ hf,
-    const float* __restrict__ a_f, const float2* __restrict__ lr_f,
-    const MixedTheta* __restrict__ theta_f, double* __restrict__ scratch)
+__global__ void __launch_bounds__(kStatsThreads) k_prep_stats(
+    const Seg* __restrict__ segs, const SerInfo* __restrict__ ser, const double* __restrict__ h,
+    const double* __restrict__ y, const double* __restrict__ lnrv, float2* __restrict__ hf,
+    float* __restrict__ a_f, float2* __restrict__ lr_f, const MixedTheta* __restrict__ theta_f,
+    double* __restrict__ scratch, unsigned* __restrict__ ser_cnt, StatsRec* __restrict__ rstats)
 {
     __shared__ float2 s_tab[32];
     __shared__ float2 s_red[kStatsThreads / 32][kPartialWords];
+    __shared__ float2 s_sum[kPartialWords];
+    __shared__ int s_last;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (tid < 32) s_tab[tid] = g_exptab[tid];
     __syncthreads();
@@ -344,24 +382,45 @@ __global__ void __launch_bounds__(kStatsThreads) k_state_stats(
     StateStats st;
     stats_zero(st);
     ff sl = {0.f, 0.f}, sll = {0.f, 0.f};
+    // the next site's inputs are loaded ahead of this one's arithmetic
+    struct In {
+        double h, hn, y, lr;
+    };
+    auto fetch = [&](int64_t t) {
+        In q{0.0, 0.0, 0.0, 0.0};
+        if (t < g.hi) {
+            const int64_t s = si.off + t;
+            q.h = h[s];
+            if (t + 1 < si.T) q.hn = h[s + 1];
+            q.y = y[s];
+            q.lr = lnrv[s];
+        }
+        return q;
+    };
+    In q = fetch(g.lo + tid);
     for (int64_t t = g.lo + tid; t < g.hi; t += kStatsThreads) {
         const int64_t s = si.off + t;
-        const float2 hv = hf[s];
-        ff x = two_sum(hv.x, -mt.mu.hi);  // x = h - mu as the trajectory kernel forms it
-        x.lo += hv.y - mt.mu.lo;
+        const In p = q;
+        q = fetch(t + kStatsThreads);
+        const ff hv = ff_split(p.h), lr = ff_split(p.lr);
+        const float as = signed_half_square(p.y);
+        hf[s] = make_float2(hv.hi, hv.lo);
+        lr_f[s] = make_float2(lr.hi, lr.lo);
+        a_f[s] = as;
+        ff x = two_sum(hv.hi, -mt.mu.hi);  // x = h - mu as the trajectory kernel forms it
+        x.lo += hv.lo - mt.mu.lo;
         x = fast_two_sum(x.hi, x.lo);
         const bool has_next = t + 1 < si.T;
         ff xn = {0.f, 0.f};
         if (has_next) {
-            const float2 hn = hf[s + 1];
-            xn = two_sum(hn.x, -mt.mu.hi);
-            xn.lo += hn.y - mt.mu.lo;
+            const ff hn = ff_split(p.hn);
+            xn = two_sum(hn.hi, -mt.mu.hi);
+            xn.lo += hn.lo - mt.mu.lo;
             xn = fast_two_sum(xn.hi, xn.lo);
         }
-        const float2 lr = lr_f[s];
-        stats_site(st, x, xn, has_next, ff{lr.x, lr.y}, fabsf(a_f[s]), mt, s_tab);
-        ff_acc(sl, ff{lr.x, lr.y});
-        ff_acc(sll, ff_mul(ff{lr.x, lr.y}, ff{lr.x, lr.y}));
+        stats_site(st, x, xn, has_next, lr, fabsf(as), mt, s_tab);
+        ff_acc(sl, lr);
+        ff_acc(sll, ff_mul(lr, lr));
         if (t == 0) st.x0 = x;
         if (t + 1 == si.T) st.xT = x;
     }
@@ -377,43 +436,47 @@ __global__ void __launch_bounds__(kStatsThreads) k_state_stats(
         ff r = {0.f, 0.f};
         for (int w = 0; w < kStatsThreads / 32; ++w)
             r = ff_add(r, ff{s_red[w][tid].x, s_red[w][tid].y});
-        float2* out = reinterpret_cast<float2*>(scratch) + (int64_t)blockIdx.x * kPartialWords;
-        out[tid] = make_float2(r.hi, r.lo);
+        s_sum[tid] = make_float2(r.hi, r.lo);
+        if (si.nseg > 1) {
+            reinterpret_cast<float2*>(scratch)[(int64_t)blockIdx.x * kPartialWords + tid] = s_sum[tid];
+            __threadfence();
+        }
     }
-}
-__global__ void k_stats_combine(const SerInfo* __restrict__ ser, int n,
-                                const MixedTheta* __restrict__ theta_f,
-                                const double* __restrict__ scratch, StatsRec* __restrict__ rstats)
-{
-    // one warp per series: lane l adds tiles l, l + 32, ... in order, then a
-    // butterfly per value
-    const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (s >= n) return;
-    const SerInfo si = ser[s];
-    const float2* rec = reinterpret_cast<const float2*>(scratch);
-    ff acc[kPartialWords];
+    __syncthreads();
+    if (si.nseg > 1) {
+        if (tid == 0) s_last = atomicAdd(ser_cnt + g.series, 1u) == (unsigned)si.nseg - 1u;
+        __syncthreads();
+        if (!s_last) return;
+        __threadfence();
+        if (tid == 0) ser_cnt[g.series] = 0u;
+        const float2* rec = reinterpret_cast<const float2*>(scratch) + (int64_t)si.seg0 * kPartialWords;
+        if (warp < kPartialWords) {  // warp k adds value k
+            ff acc = {0.f, 0.f};
+            for (int i0 = lane; i0 < si.nseg; i0 += 32 * 8) {
+                float2 v[8];
 #pragma unroll
-    for (int k = 0; k < kPartialWords; ++k) acc[k] = ff{0.f, 0.f};
-    for (int i = lane; i < si.nseg; i += 32) {
-        const float2* w = rec + (int64_t)(si.seg0 + i) * kPartialWords;
-        float2 v[kPartialWords];
+                for (int u = 0; u < 8; ++u)
+                    v[u] = i0 + 32 * u < si.nseg
+                               ? __ldcg(rec + (int64_t)(i0 + 32 * u) * kPartialWords + warp)
+                               : make_float2(0.f, 0.f);
 #pragma unroll
-        for (int k = 0; k < kPartialWords; ++k) v[k] = w[k];
-#pragma unroll
-        for (int k = 0; k < kPartialWords; ++k) acc[k] = ff_add(acc[k], ff{v[k].x, v[k].y});
+                for (int u = 0; u < 8; ++u)
+                    if (i0 + 32 * u < si.nseg) acc = ff_add(acc, ff{v[u].x, v[u].y});
+            }
+            acc = warp_sum_ff(acc);
+            if (lane == 0) s_sum[warp] = make_float2(acc.hi, acc.lo);
+        }
+        __syncthreads();
     }
-#pragma unroll
-    for (int k = 0; k < kPartialWords; ++k) acc[k] = warp_sum_ff(acc[k]);
-    if (lane == 0) {
+    if (tid == 0) {
         StatsRec r;
-        r.sl = acc[0];
-        r.sll = acc[1 + kStatsFF];
+        r.sl = ff{s_sum[0].x, s_sum[0].y};
+        r.sll = ff{s_sum[1 + kStatsFF].x, s_sum[1 + kStatsFF].y};
 #pragma unroll
-        for (int k = 0; k < kStatsFF; ++k) stats_ff(r.s)[k] = acc[1 + k];
-        r.mu = theta_f[s].mu;
-        r.ximu = theta_f[s].ximu;
-        rstats[2 * (int64_t)s] = r;
+        for (int k = 0; k < kStatsFF; ++k) stats_ff(r.s)[k] = ff{s_sum[1 + k].x, s_sum[1 + k].y};
+        r.mu = mt.mu;
+        r.ximu = mt.ximu;
+        rstats[2 * (int64_t)g.series] = r;
     }
 }
 
@@ -576,17 +639,13 @@ cudaError_t launch_traj(const TrajArgs& a, const Plan& p, cudaStream_t st)
 #undef RSV_CASE
 }
 
-cudaError_t launch_state_stats(const Plan& p, const float2* hf, const float* a_f,
-                               const float2* lr_f, const MixedTheta* theta_f, double* scratch,
-                               StatsRec* rstats, cudaStream_t st)
+cudaError_t launch_prep_stats(const Plan& p, const double* h, const double* y, const double* lnrv,
+                              float2* hf, float* a_f, float2* lr_f, const MixedTheta* theta_f,
+                              double* scratch, unsigned* ser_cnt, StatsRec* rstats, cudaStream_t st)
 {
     if (p.nsegs < 1 || p.nsegs > 0x7fffffff) return cudaErrorInvalidValue;
-    k_state_stats<<<(unsigned)p.nsegs, kStatsThreads, 0, st>>>(p.d_segs, p.d_ser, hf, a_f, lr_f,
-                                                               theta_f, scratch);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_stats_combine<<<(p.nseries + 7) / 8, 256, 0, st>>>(p.d_ser, p.nseries, theta_f, scratch,
-                                                        rstats);
+    k_prep_stats<<<(unsigned)p.nsegs, kStatsThreads, 0, st>>>(p.d_segs, p.d_ser, h, y, lnrv, hf, a_f,
+                                                              lr_f, theta_f, scratch, ser_cnt, rstats);
     return cudaGetLastError();
 }
 cudaError_t launch_commit_fp64(double* h, const double* hprop, double* p, const double* pprop,
@@ -595,10 +654,10 @@ cudaError_t launch_commit_fp64(double* h, const double* hprop, double* p, const 
     k_commit_fp64<<<grid_for(T), 256, 0, st>>>(h, hprop, p, pprop, acc, T);
     return cudaGetLastError();
 }
-cudaError_t launch_prep_mixed(const double* y, const double* lnrv, float* a_f, float2* lr_f,
-                              int64_t T, cudaStream_t st)
+cudaError_t launch_prep_mixed(const double* h, const double* y, const double* lnrv, float2* hf,
+                              float* a_f, float2* lr_f, int64_t T, cudaStream_t st)
 {
-    k_prep_mixed<<<grid_for(T), 256, 0, st>>>(y, lnrv, a_f, lr_f, T);
+    k_prep_mixed<<<grid_for(T), 256, 0, st>>>(h, y, lnrv, hf, a_f, lr_f, T);
     return cudaGetLastError();
 }
 cudaError_t launch_h_to_ff(const double* h, float2* hf, int64_t T, cudaStream_t st)
@@ -609,8 +668,13 @@ cudaError_t launch_h_to_ff(const double* h, float2* hf, int64_t T, cudaStream_t 
 cudaError_t launch_finalize(const Plan& p, const int* cur, const int* acc, const double* h1d,
                             const float2* h0f, const float2* h1f, double* h, cudaStream_t st)
 {
-    k_finalize<<<grid_for(p.total), 256, 0, st>>>(p.d_ser, p.nseries, p.total, cur, acc, h1d,
-                                                   h0f, h1f, h);
+    // segments of several series; equal runs where one series has few of them
+    const int run = 1024;
+    const bool by_seg = p.nseries > 1;
+    const int64_t g = by_seg ? p.nsegs : (p.total + run - 1) / run;
+    if (g > 0x7fffffff) return cudaErrorInvalidValue;
+    k_finalize<<<(unsigned)g, 256, 0, st>>>(by_seg ? p.d_segs : nullptr, p.d_ser, p.total, run, cur,
+                                            acc, h1d, h0f, h1f, h);
     return cudaGetLastError();
 }
 cudaError_t launch_snapshot(const Plan& p, const int* cur, const double* h0d, const double* h1d,

@@ -323,16 +323,19 @@ int mixed_max_threads(int j, bool mass);
 // Resident blocks per SM of a trajectory kernel configuration (0 if invalid).
 int blocks_per_sm(bool mixed, bool mass, bool lev, int j, int nt, size_t smem);
 
-// rstats[s][0] = the statistics of series s in the (hi, lo) state hf, for
-// every series of a mixed plan (scratch: kPartialWords doubles per segment).
-cudaError_t launch_state_stats(const Plan& p, const float2* hf, const float* a_f,
-                               const float2* lr_f, const MixedTheta* theta_f, double* scratch,
-                               StatsRec* rstats, cudaStream_t st);
+// Mixed plan without leverage, from the caller's FP64 h, y, lnRV: hf and lr_f as
+// (hi, lo) pairs, a_f = y^2/2 with the sign of y, and rstats[s][0] = the
+// statistics of series s in hf (scratch: kPartialWords doubles per segment;
+// ser_cnt: zero, and zero again afterwards).
+cudaError_t launch_prep_stats(const Plan& p, const double* h, const double* y, const double* lnrv,
+                              float2* hf, float* a_f, float2* lr_f, const MixedTheta* theta_f,
+                              double* scratch, unsigned* ser_cnt, StatsRec* rstats, cudaStream_t st);
 
 cudaError_t launch_commit_fp64(double* h, const double* hprop, double* p, const double* pprop,
                                const int* acc, int64_t T, cudaStream_t st);
-cudaError_t launch_prep_mixed(const double* y, const double* lnrv, float* a_f, float2* lr_f,
-                              int64_t T, cudaStream_t st);
+// hf, a_f and lr_f alone (the leverage model keeps no statistics).
+cudaError_t launch_prep_mixed(const double* h, const double* y, const double* lnrv, float2* hf,
+                              float* a_f, float2* lr_f, int64_t T, cudaStream_t st);
 cudaError_t launch_h_to_ff(const double* h, float2* hf, int64_t T, cudaStream_t st);
 // Write the current state of every series into h (packed FP64): FP64 path
 // from h1d where cur[s] = 1 (h0d is h itself); mixed path from the (hi, lo)
