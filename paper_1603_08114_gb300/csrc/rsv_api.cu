@@ -168,7 +168,7 @@ rsv_status rsv_reserve(rsv_ctx* c, int64_t max_T, int64_t max_series)
     if ((st = c->ser_acc.ensure(n * sizeof(int))) != RSV_OK) return st;
     if ((st = c->theta_f.ensure(n * sizeof(MixedTheta))) != RSV_OK) return st;
     if ((st = c->rstats.ensure(n * 2 * sizeof(StatsRec))) != RSV_OK) return st;
-    if ((st = c->gibbs.ensure((size_t)gibbs_grid(max_T) * 8 * sizeof(double))) != RSV_OK) return st;
+    if ((st = c->gibbs.ensure(gibbs_scratch(max_T))) != RSV_OK) return st;
     return RSV_OK;
 }
 
@@ -255,7 +255,7 @@ rsv_status rsv_action(rsv_ctx* c, const double* h, const double* y, const double
     if (!h || !y || !lnrv || !S_out) return fail(RSV_EINVAL, "null array argument");
     if (T < 1) return fail(RSV_EINVAL, "T must be >= 1 (got %lld)", (long long)T);
     if (!theta_ok(theta)) return fail(RSV_EINVAL, "invalid theta");
-    if ((st = ctx_ensure_partials(c, action_grid(T))) != RSV_OK) return st;
+    if ((st = c->partials.ensure((size_t)action_grid(T) * sizeof(double))) != RSV_OK) return st;
     ThetaD th = to_dev(theta);
     th.rho = c->rho;
     cudaError_t e = counted(c, launch_action, h, y, lnrv, T, th, c->partials.as<double>(),
@@ -305,7 +305,7 @@ rsv_status rsv_gibbs_theta(rsv_ctx* c, const double* h, const double* lnrv, int6
     if (c->rho != 0.0)
         return fail(RSV_EINVAL, "the theta update is for the model without leverage (rho = 0)");
     const bool mixed = prec == RSV_MIXED;
-    if ((st = c->gibbs.ensure((size_t)gibbs_grid(T) * 8 * sizeof(double))) != RSV_OK) return st;
+    if ((st = c->gibbs.ensure(gibbs_scratch(T))) != RSV_OK) return st;
     if (mixed && ((st = c->fbuf0.ensure((size_t)T * 8)) != RSV_OK ||
                   (st = c->lr_f.ensure((size_t)T * 8)) != RSV_OK ||
                   (st = c->theta_f.ensure(sizeof(MixedTheta))) != RSV_OK))

@@ -200,7 +200,7 @@ rsv_status run(rsv_ctx* c, const Plan& P, const RunOpts& o, cudaStream_t s)
     rsv_status st;
     if ((st = ensure_plan_ws(c, P, mixed, o.p != nullptr)) != RSV_OK) return st;
     if (o.update_theta &&
-        (st = c->gibbs.ensure((size_t)gibbs_grid(P.total) * 8 * sizeof(double))) != RSV_OK)
+        (st = c->gibbs.ensure(gibbs_scratch(P.total))) != RSV_OK)
         return st;
     int* ints = c->ints.as<int>();
     cudaError_t e;

@@ -287,9 +287,15 @@ __device__ __forceinline__ void exp_table(u64* tab)
         tab[i] = (hi << 1) + (lo >> 63) + ((lo >> 62) & 1);  // the product in units of 2^-63, rounded
     }
 }
+// The two small tables alone, for launches too short to be worth kExpN products:
+// exp_neg<.., .., true> multiplies their entries at each evaluation.
+__device__ __forceinline__ void exp_table_small(u64* tab)
+{
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) tab[i] = i < 32 ? kExpHi[i] : kExpLo[i - 32];
+}
 static __device__ __noinline__ double exp_slow(double a) { return exp(a); }
-// e^{-x / 2^SH} (SH = 0 or 1; the halving is exact)
-template <int SH = 0>
+// e^{-x / 2^SH} / 2^HALF (SH, HALF = 0 or 1; both halvings are exact)
+template <int SH = 0, int HALF = 0, bool SMALL = false>
 __device__ __forceinline__ double exp_neg(double x, const u64* tab)
 {
     const unsigned xh = (unsigned)__double2hiint(x), xl = (unsigned)__double2loint(x);
@@ -310,16 +316,23 @@ __device__ __forceinline__ double exp_neg(double x, const u64* tab)
     const unsigned w = __umulhi(rr, 174763u) + 0x2aaaaaabu;        // 1/6 + r/24, 2^-32
     const u64 P = R + (r2 >> 19) + (__umulhi(rr, (unsigned)R << 8) >> 18) +
                   ((u64)__umulhi(c, w) << 4);                      // p, 2^-66
-    const u64 T = tab[k & (kExpN - 1)];
+    u64 T;
+    if (SMALL) {
+        const u64 a = tab[(k >> 5) & 31], b = tab[32 + (k & 31)];
+        const u64 hi = __umul64hi(a, b), lo = a * b;
+        T = (hi << 1) + (lo >> 63) + ((lo >> 62) & 1);
+    } else {
+        T = tab[k & (kExpN - 1)];
+    }
     const unsigned Th = (unsigned)(T >> 32), Tl = (unsigned)T;
     const unsigned Ph = (unsigned)(P >> 32), Pl = (unsigned)P;
     const u64 tp = (u64)Th * Ph + __umulhi(Th, Pl) + __umulhi(Tl, Ph);  // T p, 2^-65
     const u64 m = T + (tp >> 2);
     // a negative r, a carry out of m (bit 63 is set otherwise) or |a| >= 128
     if (((int)(R >> 32) | (int)~(unsigned)(m >> 32) | sh) < 0)
-        return exp_slow(SH ? -0.5 * x : -x);
+        return (HALF ? 0.5 : 1.0) * exp_slow(SH ? -0.5 * x : -x);
     const u64 v = (m >> 11) + ((m >> 10) & 1);
-    return __longlong_as_double((long long)(v + ((u64)(unsigned)((k >> 10) + 1022) << 52)));
+    return __longlong_as_double((long long)(v + ((u64)(unsigned)((k >> 10) + 1022 - HALF) << 52)));
 }
 
 // ---------------------------------------------------------------------------
@@ -357,6 +370,30 @@ __device__ __forceinline__ double block_sum(double v, double* red)
         s = warp_sum(s);
     }
     return s;
+}
+
+// Block sums of N values (blockDim.x = NT threads, NT / 32 >= N warps): warp i
+// adds value i over the threads, lane l those of l, l + 32, ... in order, then
+// a butterfly (a butterfly per warp and value first would take five of the FP64
+// pipe's instructions for each one that this takes).  tot[i] is valid in every
+// thread after the call.
+template <int N, int NT>
+__device__ __forceinline__ void block_sum_many(const double (&v)[N], double (*buf)[NT], double* tot)
+{
+    static_assert(NT / 32 >= N, "one warp per value");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < N; ++i) buf[i][threadIdx.x] = v[i];
+    __syncthreads();
+    if (warp < N) {
+        double s = buf[warp][lane];
+#pragma unroll
+        for (int k = 1; k < NT / 32; ++k) s += buf[warp][lane + 32 * k];
+        s = warp_sum(s);
+        if (lane == 0) tot[warp] = s;
+    }
+    __syncthreads();
 }
 
 // Theta as stored on the device: (phi, mu, xi, sigma_eta^2, sigma_u^2), and

@@ -1,6 +1,7 @@
 // rsv_gibbs.cuh -- launcher of the theta Gibbs sweep.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -21,7 +22,7 @@ struct GibbsArgs {
     double* theta_out;   // optional record [5]
     uint64_t seed, series, traj;
     int mask;            // components updated: bit 0 xi .. bit 4 phi
-    double* partials;    // [grid * 8]
+    double* partials;    // gibbs_scratch(T) bytes
     unsigned* counter;
     int* phi_acc;        // optional
     MixedTheta* theta_f; // mixed path: the current theta's constants, read and refreshed
@@ -32,7 +33,8 @@ struct GibbsArgs {
     const StatsRec* rstats;
 };
 
-int gibbs_grid(int64_t T);
+// Bytes of scratch a sweep of T sites needs.
+size_t gibbs_scratch(int64_t T);
 cudaError_t launch_gibbs(const GibbsArgs& a, bool mixed, cudaStream_t st);
 
 }  // namespace rsv
