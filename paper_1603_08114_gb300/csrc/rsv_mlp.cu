@@ -452,16 +452,30 @@ __device__ __forceinline__ void mlp_group(StepSmem& S, const Fetch& q, const Ste
         part[i] = ((S.grad[0][i] + S.grad[1][i]) + S.grad[2][i]) + S.grad[3][i];
 }
 
-// Adam (Kingma & Ba 2015) of parameter i with gradient g, FP32; time t.
-__device__ __forceinline__ void adam_step(const StepArgs& A, int i, float g, int64_t t)
+// Adam (Kingma & Ba 2015) of parameter i with gradient g, FP32; c1 = 1 - b1^t
+// and c2 = 1 - b2^t of the step's time t.
+struct AdamState {
+    float m, v, p;
+};
+__device__ __forceinline__ AdamState adam_load(const StepArgs& A, int i)
 {
-    const float m = A.b1 * __ldcg(A.adam_m + i) + (1.f - A.b1) * g;
-    const float v = A.b2 * __ldcg(A.adam_v + i) + (1.f - A.b2) * g * g;
+    return AdamState{__ldcg(A.adam_m + i), __ldcg(A.adam_v + i), __ldcg(A.params + i)};
+}
+__device__ __forceinline__ void adam_step(const StepArgs& A, int i, float g, float c1, float c2,
+                                          const AdamState& q)
+{
+    const float m = A.b1 * q.m + (1.f - A.b1) * g;
+    const float v = A.b2 * q.v + (1.f - A.b2) * g * g;
     A.adam_m[i] = m;
     A.adam_v[i] = v;
-    const float mh = m / (1.f - powf(A.b1, (float)t));
-    const float vh = v / (1.f - powf(A.b2, (float)t));
-    A.params[i] = __ldcg(A.params + i) - A.lr * mh / (sqrtf(vh) + A.eps);
+    const float mh = m / c1;
+    const float vh = v / c2;
+    A.params[i] = q.p - A.lr * mh / (sqrtf(vh) + A.eps);
+}
+__device__ __forceinline__ void adam_corrections(const StepArgs& A, int64_t t, float& c1, float& c2)
+{
+    c1 = 1.f - powf(A.b1, (float)t);
+    c2 = 1.f - powf(A.b2, (float)t);
 }
 
 // One minibatch in one launch, a block per group of 64 sites: loss and
@@ -489,6 +503,8 @@ __global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
     __syncthreads();
     if (!s_last) return;
     __threadfence();
+    float c1 = 1.f, c2 = 1.f;
+    if (A.update) adam_corrections(A, A.adam_t, c1, c2);
     for (int i = tid; i < NPARAM + 1; i += blockDim.x) {
         float s = 0.f;
 #pragma unroll 16
@@ -499,7 +515,7 @@ __global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
             continue;
         }
         if (A.grad_out) A.grad_out[i] = s;
-        if (A.update) adam_step(A, i, s, A.adam_t);
+        if (A.update) adam_step(A, i, s, c1, c2, adam_load(A, i));
     }
     if (tid == 0) *A.counter = 0u;
 }
@@ -511,7 +527,8 @@ __global__ void __launch_bounds__(128) k_mlp_step(const StepArgs A)
 // group's gradient, a grid barrier, then each adds the partials of its own
 // slice of the parameters (block order, as the step kernel) and takes their
 // Adam step, a second barrier.  The next minibatch's sites are fetched while
-// the first barrier is waited for.  Batch 4096: 53 -> 9.0 us a step.
+// the first barrier is waited for.  Batch 4096: 53 -> 7.9 us a step, batch 64 (one
+// block) 27 -> 10.
 struct GridBarrier {
     unsigned* bar;
     unsigned target;
@@ -572,8 +589,13 @@ __global__ void __launch_bounds__(128) k_mlp_train(const StepArgs A)
         gb.arrive(nb);
         if (n + 1 < A.n_steps) fetch_sites(A, A.step + n + 1, k0, q);
         if (!gb.wait(A.wait_limit, A.status, &s_ok)) return;
-        for (int c = lo; c < hi; c += 32) {
-            const int i = c + lane;
+        float c1, c2;
+        adam_corrections(A, A.adam_t + n, c1, c2);
+        if (per <= 32) {
+            // one parameter a lane: four warps stage the rows, one adds them
+            const int i = lo + lane;
+            AdamState q{0.f, 0.f, 0.f};
+            if (warp == 0 && i < hi && i < NPARAM) q = adam_load(A, i);
             float s = 0.f;
             for (int r0 = 0; r0 < nb; r0 += kRedRows) {
                 const int rows = min(kRedRows, nb - r0);
@@ -589,8 +611,46 @@ __global__ void __launch_bounds__(128) k_mlp_train(const StepArgs A)
                 }
             }
             if (warp == 0 && i < hi) {
-                if (i < NPARAM) adam_step(A, i, s, A.adam_t + n);
+                if (i < NPARAM) adam_step(A, i, s, c1, c2, q);
                 else if (A.loss_out) A.loss_out[n] = s / (float)A.batch;
+            }
+        } else if (per <= 128) {
+            // one parameter a thread
+            const int i = lo + tid;
+            if (i < hi) {
+                AdamState q{0.f, 0.f, 0.f};
+                if (i < NPARAM) q = adam_load(A, i);
+                float s = 0.f;
+#pragma unroll 16
+                for (int r = 0; r < nb; ++r)
+                    s += __ldcg(A.partials + (int64_t)r * (NPARAM + 1) + i);
+                if (i < NPARAM) adam_step(A, i, s, c1, c2, q);
+                else if (A.loss_out) A.loss_out[n] = s / (float)A.batch;
+            }
+        } else {
+            // few blocks, many parameters each: kU a thread at a time over few rows
+            constexpr int kU = 7;
+            for (int i0 = lo + tid; i0 < hi; i0 += 128 * kU) {
+                float s[kU];
+                AdamState q[kU];
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int i = i0 + 128 * u;
+                    s[u] = 0.f;
+                    if (i < hi && i < NPARAM) q[u] = adam_load(A, i);
+                }
+                for (int r = 0; r < nb; ++r)
+#pragma unroll
+                    for (int u = 0; u < kU; ++u)
+                        if (i0 + 128 * u < hi)
+                            s[u] += __ldcg(A.partials + (int64_t)r * (NPARAM + 1) + i0 + 128 * u);
+#pragma unroll
+                for (int u = 0; u < kU; ++u) {
+                    const int i = i0 + 128 * u;
+                    if (i >= hi) continue;
+                    if (i < NPARAM) adam_step(A, i, s[u], c1, c2, q[u]);
+                    else if (A.loss_out) A.loss_out[n] = s[u] / (float)A.batch;
+                }
             }
         }
         if (n + 1 == A.n_steps) return;
