@@ -44,9 +44,9 @@ cudaError_t timed_traj(rsv_ctx* c, const TrajArgs& a, const Plan& p, cudaStream_
     return e;
 }
 
-// Single-series plan from the context cache.  chain: the plan of an
-// rsv_hmc_chain call that can run as one persistent launch (its own block
-// shape preference).
+// Single-series plan from the context cache.  chain: the plan of a mixed
+// rsv_hmc_chain call (its own block shape preference; without leverage it can
+// run as one persistent launch).
 rsv_status single_plan(rsv_ctx* c, int64_t T, int n_md, bool mixed, bool mass, const Plan** out,
                        bool chain = false)
 {
@@ -416,7 +416,7 @@ rsv_status rsv_hmc_chain(rsv_ctx* c, double* h, const double* y, const double* l
     if (update_theta && c->rho != 0.0)
         return fail(RSV_EINVAL, "the theta update is for the model without leverage (rho = 0)");
     const Plan* P = nullptr;
-    const bool chain = prec == RSV_MIXED && c->rho == 0.0 && c->persistent;
+    const bool chain = prec == RSV_MIXED && c->persistent;  // a chain's block shape
     if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, minv != nullptr, &P, chain)) != RSV_OK)
         return st;
     RunOpts o;
@@ -450,12 +450,12 @@ rsv_status rsv_chain_schedule(rsv_ctx* c, int64_t T, int n_md, rsv_precision pre
     if (st != RSV_OK) return st;
     if (T < 1) return fail(RSV_EINVAL, "T must be >= 1 (got %lld)", (long long)T);
     if ((st = check_common(n_md, 1.0, prec)) != RSV_OK) return st;
-    const bool chain = prec == RSV_MIXED && c->rho == 0.0 && c->persistent;
+    const bool chain = prec == RSV_MIXED && c->persistent;
     const Plan* P = nullptr;
     if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, with_mass != 0, &P, chain)) != RSV_OK)
         return st;
     bool fits = false;
-    if (chain) {
+    if (chain && c->rho == 0.0) {
         cudaError_t e = chain_fits(*P, c->num_sms, &fits);
         if (e != cudaSuccess) return cuda_fail(e, "chain occupancy");
     }

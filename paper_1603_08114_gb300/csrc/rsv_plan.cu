@@ -48,22 +48,67 @@ bool valid_j(bool mixed, int j)
     return false;
 }
 
-// Time in us of one FP64 trajectory of a single series as `bins` blocks of nt
-// threads with j sites each, n_force force evaluations, of which bps fit on an
-// SM.  A step is the longer of one warp's own latency (0.30 + 0.36 j) and the
-// SM's FP64 pipe, which all its warps share (0.50 + 0.0625 j per warp); a
-// launch's draws, energies and decision about 16 + 3 j.  Fitted to a sweep of
-// every shape (32 .. 256 threads, j = 1 .. 28) at T = 500 .. 2^18 and n_md = 10
-// .. 80, off by 10 % at most near the optimum: T = 2000, 50 steps 46 us (87 blocks of
-// 128 x 1) against 121 us (4 blocks of 192 x 4, the fewest sites in flight),
-// T = 30000, 50 steps 72 us (160 x 2) against 106 us (128 x 4).
-double fp64_cost(int64_t bins, int nt, int j, int n_force, int num_sms, int bps)
+// Time in us of one round of a trajectory -- the blocks an SM holds at once,
+// with `warps` warps of j sites per thread between them, through n_force force
+// evaluations -- as fitted to sweeps of every block shape.
+//
+// FP64 (T = 500 .. 2^18, 10 .. 80 steps): a step is the longer of one warp's own
+// latency (0.30 + 0.36 j) and the SM's FP64 pipe, which all its warps share (0.50
+// + 0.0625 j per warp); the draws, energies and decision take about 16 + 3 j.
+// Off by 10 % at most near the optimum: T = 2000, 50 steps 46 us (87 blocks of
+// 128 x 1) against 121 us (4 blocks of 192 x 4, the fewest sites in flight), T =
+// 30000, 50 steps 72 us (160 x 2) against 106 us (128 x 4).
+//
+// Mixed (persistent chains of T = 500 .. 2^20, 10 .. 100 steps, theta sampled): a
+// step has a latency that grows with j up to four warps and then with every
+// further warp; so has the fixed part.  T = 2000, 50 steps 20.8 us a trajectory
+// (5 blocks of 128 x 4) against 33.0 (one block of 544 x 4), T = 30000 21.4
+// (74 of 128 x 4) against 33.0, T = 700000, 90 steps 66 (142 of 640 x 8)
+// against 72 (256 x 20); at 2^20 sites only the windows of 384 x 20 fit in one
+// round of 12 warps (87 us with 78 steps and a mass; 448 x 16: 90, 608 x 12:
+// 94).  With leverage a step takes about 1.4 times as long.
+double round_cost(bool mixed, bool lev, int j, double warps, double n_force)
 {
-    const int64_t per = std::min<int64_t>(bps, (bins + num_sms - 1) / num_sms);
-    const int64_t waves = (bins + per * num_sms - 1) / (per * num_sms);
-    const double warps = (double)per * (nt / 32);
-    const double step = std::max(0.30 + 0.36 * j, 0.50 + 0.0625 * j * warps);
-    return waves * (16.0 + 3.0 * j + n_force * step) * (1.0 + 1e-6 * bins);
+    if (!mixed)
+        return 16.0 + 3.0 * j + n_force * std::max(0.30 + 0.36 * j, 0.50 + 0.0625 * j * warps);
+    const double more = std::max(0.0, warps - 4.0);
+    double step, fixed;
+    switch (j) {
+        case 4: step = 0.147 + 0.0119 * more, fixed = 13.3 + 0.22 * warps; break;
+        case 8: step = 0.21 + 0.0195 * more, fixed = 16.0 + 0.22 * warps; break;
+        case 12: step = 0.32 + 0.031 * more, fixed = 20.0 + 0.55 * warps; break;
+        case 16: step = 0.305 + 0.045 * more, fixed = 19.9 + 0.7 * warps; break;
+        default: step = 0.36 + 0.038 * more, fixed = 19.1 + 0.9 * warps; break;
+    }
+    return fixed + n_force * step * (lev ? 1.4 : 1.0);
+}
+
+// Bins that whole series of cnt[w] x w warps need at NW warps a bin, larger
+// ones first, each into the fullest bin with room (an estimate of the packing
+// below, which takes the first such bin).
+int64_t packed_bins(const std::vector<int64_t>& cnt, int NW)
+{
+    std::vector<int64_t> room(NW + 1, 0);  // bins by the warps they have left
+    int64_t bins = 0;
+    for (int w = NW; w >= 1; --w) {
+        int64_t left = cnt[w];
+        for (int r = w; r <= NW && left > 0; ++r) {
+            while (room[r] > 0 && left > 0) {
+                const int64_t per = r / w, use = std::min(room[r], (left + per - 1) / per);
+                const int64_t put = std::min(left, use * per);
+                const int64_t full = put / per, rest = put % per;
+                room[r] -= full + (rest ? 1 : 0);
+                room[r - per * w] += full;
+                if (rest) room[r - rest * w] += 1;
+                left -= put;
+            }
+        }
+        const int64_t per = NW / w, full = left / per, rest = left % per;
+        bins += full + (rest ? 1 : 0);
+        room[NW - per * w] += full;
+        if (rest) room[NW - rest * w] += 1;
+    }
+    return bins;
 }
 
 int ntmax(bool mixed, bool mass, int j) { return mixed ? mixed_max_threads(j, mass) : 256; }
@@ -157,27 +202,26 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                     if (bps < 1) continue;
                     const int64_t waves = (b + (int64_t)num_sms * bps - 1) / ((int64_t)num_sms * bps);
                     double cost = (double)waves * (double)cap * bps;
-                    if (!mixed) cost = fp64_cost(b, t, js[ji], (int)(K - 1), num_sms, bps);
-                    // measured on the mixed kernel at T = 2^20 (fixed and
-                    // per-step cost per block shape): J = 12 with ~600
-                    // threads is the fastest, J = 20 close, J = 16 and 8
-                    // slower; inside the persistent chain (78 steps, mass,
-                    // every state recorded) J = 20 with 384 threads is the
-                    // fastest, 89.5 us per trajectory against 92.1 for
-                    // J = 16 (448 threads) and 91.9 for J = 12 (608): per
-                    // site of a window 0.0117, 0.0128 and 0.0126 us
-                    if (mixed && chain)
-                        cost *= js[ji] == 20 ? 0.91 : js[ji] == 16 ? 1.0 : js[ji] == 12 ? 0.98 : 1.1;
-                    else if (mixed)
+                    if (!mixed) {
+                        const int64_t per = std::min<int64_t>(bps, (b + num_sms - 1) / num_sms);
+                        cost = (double)((b + per * num_sms - 1) / (per * num_sms)) *
+                               round_cost(false, lev, js[ji], (double)per * (t / 32), (double)(K - 1)) *
+                               (1.0 + 1e-6 * b);
+                    } else if (chain) {
+                        // one block per SM: a round more is a launch more
+                        const int64_t w = (b + num_sms - 1) / num_sms;
+                        cost = (double)w * (round_cost(true, lev, js[ji], t / 32, (double)(K - 1)) +
+                                            (w > 1 ? 6.0 : 0.0)) + 0.005 * b;
+                    }
+                    // single trajectories (mixed): measured at T = 2^20, J = 12
+                    // with ~600 threads is the fastest, J = 20 close, J = 16 and
+                    // 8 slower; a series cut into tiles runs at the throughput
+                    // of its blocks, which falls with fewer warps, a whole one
+                    // keeps the smallest window (a tie-break toward more threads)
+                    if (mixed && !chain) {
                         cost *= js[ji] == 12 ? 1.0 : js[ji] == 20 ? 1.03 : 1.08;
-                    // a series cut into tiles runs at the throughput of
-                    // its blocks, which falls with fewer warps (the
-                    // leapfrog is latency-bound): measured on the mixed
-                    // kernel at T = 2^22, 384 x 20 takes 0.382 ms a
-                    // trajectory in 4 waves, 288 x 20 0.449 ms in 5 (25 %
-                    // more per site); a whole series keeps the smallest
-                    // window (a tie-break toward more threads only)
-                    if (mixed) cost *= 1.0 + (b > 1 ? 1.0 : 1e-3) * (double)(tmax - t) / tmax;
+                        cost *= 1.0 + (b > 1 ? 1.0 : 1e-3) * (double)(tmax - t) / tmax;
+                    }
                     if (cost < best) {
                         best = cost;
                         nt = t;
@@ -192,11 +236,60 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
             return false;
         }
     } else {
-        // many series: the largest window, so that most series are whole
-        j = mixed ? 20 : 28;
-        nt = ntmax(mixed, mass, j);
-        tile = (int64_t)nt * j - 2 * K - 3;
-        if (tile < 1) {
+        // many series: the shape with the least estimated time, in rounds of the
+        // bins an SM holds at once.  Mixed plans keep runs of 20 sites, and the
+        // largest block where a series is longer than its window, so that a
+        // series' double-float sums are taken in the same order whatever it
+        // is packed with; smaller blocks spread few short series over the SMs
+        // (10 series of 300 .. 1000 sites, 40 steps: 64 x 20 in 7 blocks 54 us a
+        // trajectory, 384 x 20 in 2 78).  FP64 takes any run (64 series of 300
+        // .. 2000: 192 x 2 120 us a trajectory, 256 x 28 702).
+        double best = 1e300;
+        const int big_j = mixed ? 20 : 28, big_t = ntmax(mixed, mass, big_j);
+        if ((int64_t)big_t * big_j - 2 * K - 3 < 1) {
+            *why = "n_md too large for an on-chip window";
+            return false;
+        }
+        const int only[] = {20};
+        const int* js = mixed ? only : kJ_fp64;
+        const int nj = mixed ? 1 : kNJ_fp64;
+        for (int ji = 0; ji < nj; ++ji) {
+            const int tmax = ntmax(mixed, mass, js[ji]);
+            for (int t = 32; t <= tmax; t += 32) {
+                const int64_t cap = (int64_t)t * js[ji], tl = cap - 2 * K - 3, pw = 32LL * js[ji];
+                const size_t sm = smem_for(mixed, mass, lev, t, js[ji]);
+                if (sm > smem_cap || (tl < 1 && Tmax > cap)) continue;
+                if (mixed && Tmax > cap && t < tmax) continue;
+                std::vector<int64_t> cnt(t / 32 + 1, 0);
+                int64_t b = 0, segs = 0;
+                for (int s = 0; s < n; ++s) {
+                    const int64_t T = off[s + 1] - off[s];
+                    if (T <= cap) {
+                        ++cnt[(T + pw - 1) / pw];
+                        ++segs;
+                    } else {
+                        b += (T + tl - 1) / tl;
+                    }
+                }
+                segs += b;
+                // (rsv_reserve grows the partials for total / 64 + 4096 segments)
+                if (segs > off[n] / 64 + 4096) continue;
+                b += packed_bins(cnt, t / 32);
+                const int bps = blocks_per_sm(mixed, mass, lev, js[ji], t, sm);
+                if (bps < 1) continue;
+                const int64_t per = std::min<int64_t>(bps, (b + num_sms - 1) / num_sms);
+                const double cost =
+                    (double)((b + per * num_sms - 1) / (per * num_sms)) *
+                    (round_cost(mixed, lev, js[ji], (double)per * (t / 32), (double)(K - 1)) + 6.0);
+                if (cost < best) {
+                    best = cost;
+                    nt = t;
+                    j = js[ji];
+                    tile = std::max<int64_t>(tl, 1);
+                }
+            }
+        }
+        if (nt == 0) {
             *why = "n_md too large for an on-chip window";
             return false;
         }

@@ -38,7 +38,10 @@
 //   B = 1 / (s_eta^2 (1 - rho^2)),
 // and the y-term (y^2/2) e^{-h} = eps^2 / 2; the stationary term of h_1 is
 // unchanged.
+#include <array>
 #include <cmath>
+#include <map>
+#include <mutex>
 
 #include "rsv_traj_dev.cuh"
 
@@ -571,10 +574,24 @@ int mixed_max_threads(int j, bool mass)
     }
 }
 
+// The answers are kept (a property of the device and the kernel): a plan weighs
+// dozens of shapes, and a query takes several microseconds.
 int blocks_per_sm(bool mixed, bool mass, bool lev, int j, int nt, size_t smem)
 {
-    int n = 0;
-    cudaError_t e = cudaSuccess;
+    static std::mutex mu;
+    static std::map<std::array<int64_t, 5>, int> known;
+    int n = 0, dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return 0;
+    }
+    const std::array<int64_t, 5> key{dev, mixed * 4 + mass * 2 + lev, j, nt, (int64_t)smem};
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = known.find(key);
+        if (it != known.end()) return it->second;
+    }
 #define RSV_OCC(KERN)                                                                     \
     do {                                                                                  \
         e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
@@ -608,6 +625,8 @@ int blocks_per_sm(bool mixed, bool mass, bool lev, int j, int nt, size_t smem)
         (void)cudaGetLastError();
         return 0;
     }
+    std::lock_guard<std::mutex> lk(mu);
+    known[key] = n;
     return n;
 }
 
