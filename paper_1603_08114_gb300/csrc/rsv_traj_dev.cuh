@@ -479,33 +479,12 @@ __device__ __forceinline__ void mixed_steps(float2 (&X)[J / 2], float2 (&XL)[J /
         const float2 t = fma2(nl2h, xq, cmh);
         return f2(ex2_approx(t.x), ex2_approx(t.y));
     };
-    // short runs have registers to spare for their pairs' constants, which the
-    // step would otherwise wait for after its barrier (a chain of 2000 sites, 50
-    // steps: 33.0 -> 32.1 us a trajectory)
-    constexpr bool REG = J <= 4 && !LEV;
-    float4 akr[REG ? P : 1];
-    float2 dmr[REG && MASS ? P : 1];
-    if (REG) {
-#pragma unroll
-        for (int q = 0; q < (REG ? P : 0); ++q) {
-            akr[q] = s_ak[q * NTP + tid];
-            if (MASS) dmr[q] = s_dm[q * NTP + tid];
-        }
-    }
-    auto ak_of = [&](int q) -> float4 {
-        if constexpr (REG) return akr[q];
-        else return s_ak[q * NTP + tid];
-    };
-    auto dm_of = [&](int q) -> float2 {
-        if constexpr (REG && MASS) return dmr[q];
-        else return s_dm[q * NTP + tid];
-    };
     // one pair: force of eq. (7) in three-point form, then the kick and the
     // drift, compensated.  LEV: e2 = e^{-h/2} of the pair, prevw = w of its
     // left neighbours; returns the pair's w.
     auto advance = [&](int q, float2 prev, float2 nxt, float2 cx, float hs, float2 e2,
                        float2 prevw) -> float2 {
-        const float4 ak = ak_of(q);
+        const float4 ak = s_ak[q * NTP + tid];
         const float2 xq = X[q];
         if (EDGE) {
             if (q == c.la) nxt.x = c.phi * xq.x;
@@ -527,7 +506,7 @@ __device__ __forceinline__ void mixed_steps(float2 (&X)[J / 2], float2 (&XL)[J /
         }
         // with a mass the state holds the velocity v = p/m: the kick takes
         // the per-site -kick/m, the drift is the same for every site
-        const float2 km = MASS ? (KV ? fma2(dm_of(q), kc, zero) : dm_of(q))
+        const float2 km = MASS ? (KV ? fma2(s_dm[q * NTP + tid], kc, zero) : s_dm[q * NTP + tid])
                                : (KV ? kc : ndt);
         cupd2(PH[q], PL[q], km, f);
         cupd2(X[q], XL[q], cx, PH[q]);
