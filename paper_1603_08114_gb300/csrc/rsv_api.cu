@@ -160,8 +160,8 @@ rsv_status rsv_reserve(rsv_ctx* c, int64_t max_T, int64_t max_series)
     if ((st = c->fbuf1.ensure(T * 8)) != RSV_OK) return st;
     if ((st = c->a_f.ensure(T * 4)) != RSV_OK) return st;
     if ((st = c->lr_f.ensure(T * 8)) != RSV_OK) return st;
-    if ((st = ctx_ensure_partials(c, (max_T / 64 + 4096))) != RSV_OK) return st;
     const size_t n = (size_t)(max_series > 1 ? max_series : 1);
+    if ((st = ctx_ensure_partials(c, reserved_segs(max_T, (int64_t)n))) != RSV_OK) return st;
     if ((st = c->ser_cur.ensure(n * sizeof(int))) != RSV_OK) return st;
     if ((st = c->ser_cnt.ensure(n * sizeof(unsigned))) != RSV_OK) return st;
     if ((st = c->ser_dh.ensure(n * sizeof(double))) != RSV_OK) return st;

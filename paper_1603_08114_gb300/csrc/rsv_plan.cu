@@ -272,8 +272,9 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                     }
                 }
                 segs += b;
-                // (rsv_reserve grows the partials for total / 64 + 4096 segments)
-                if (segs > off[n] / 64 + 4096) continue;
+                // prefer shapes within the segments rsv_reserve grows the
+                // partials for (a whole series is one, whatever its length)
+                if (segs > reserved_segs(off[n], n)) continue;
                 b += packed_bins(cnt, t / 32);
                 const int bps = blocks_per_sm(mixed, mass, lev, js[ji], t, sm);
                 if (bps < 1) continue;
@@ -289,9 +290,10 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                 }
             }
         }
-        if (nt == 0) {
-            *why = "n_md too large for an on-chip window";
-            return false;
+        if (nt == 0) {  // tiles of a few sites in every shape: the largest window
+            nt = big_t;
+            j = big_j;
+            tile = (int64_t)big_t * big_j - 2 * K - 3;
         }
     }
     const int64_t cap = (int64_t)nt * j;

@@ -320,6 +320,10 @@ __host__ __device__ constexpr int mixed_ntp(int nt) { return nt; }
 // Largest block (threads) of the mixed kernel with `j` sites per thread, with
 // or without a mass (0 if j is not instantiated).
 int mixed_max_threads(int j, bool mass);
+// Segments that rsv_reserve grows the partials for: one per series and the
+// tiles of the cut ones, as many as a plan has unless n_md is so large that even
+// the largest window owns fewer than 64 sites.
+inline int64_t reserved_segs(int64_t total, int64_t nseries) { return total / 64 + 4096 + nseries; }
 // Resident blocks per SM of a trajectory kernel configuration (0 if invalid).
 int blocks_per_sm(bool mixed, bool mass, bool lev, int j, int nt, size_t smem);
 
