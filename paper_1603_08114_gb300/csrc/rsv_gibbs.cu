@@ -516,7 +516,8 @@ __global__ void __launch_bounds__(32) k_gibbs_stats(GibbsArgs A)
 // FP64 path: a site per thread while that leaves no SM two blocks, else runs of
 // kGibbsRun sites, up to 8 blocks per SM.  Mixed path: one wave of two blocks of
 // 256 per SM (loads of four sites in flight).
-static bool gibbs_short(int64_t T) { return T <= 152 * kGibbsThreads; }
+constexpr int64_t kGibbsShort = 152 * kGibbsThreads;
+static bool gibbs_short(int64_t T) { return T <= kGibbsShort; }
 static int gibbs_grid(int64_t T)
 {
     const int per = kGibbsThreads * (gibbs_short(T) ? 1 : kGibbsRun);
@@ -525,9 +526,13 @@ static int gibbs_grid(int64_t T)
     if (g < 1) g = 1;
     return (int)g;
 }
+// (what is enough for T sites is enough for fewer: the longest short series has
+// more blocks than a series four times as long)
 size_t gibbs_scratch(int64_t T)
 {
-    return ((size_t)gibbs_grid(T) * NSTAT + kPreWords) * sizeof(double);
+    int g = gibbs_grid(T);
+    if (!gibbs_short(T) && g < gibbs_grid(kGibbsShort)) g = gibbs_grid(kGibbsShort);
+    return ((size_t)g * NSTAT + kPreWords) * sizeof(double);
 }
 static int gibbs_grid_mixed(int64_t T)
 {

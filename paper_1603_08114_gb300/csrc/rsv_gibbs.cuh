@@ -33,7 +33,7 @@ struct GibbsArgs {
     const StatsRec* rstats;
 };
 
-// Bytes of scratch a sweep of T sites needs.
+// Bytes of scratch that a sweep of T sites, or of fewer, needs.
 size_t gibbs_scratch(int64_t T);
 cudaError_t launch_gibbs(const GibbsArgs& a, bool mixed, cudaStream_t st);
 
