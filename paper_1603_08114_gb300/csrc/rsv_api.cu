@@ -13,6 +13,7 @@
 #include "rsv_ctx.cuh"
 #include "rsv_ess.cuh"
 #include "rsv_gibbs.cuh"
+#include "rsv_mlp.cuh"
 #include "rsv_simple.cuh"
 #include "rsv_traj.cuh"
 #include "rsv_api_common.cuh"
@@ -123,6 +124,7 @@ rsv_status rsv_create(rsv_ctx** out, int device)
     g_cur_stream = nullptr;
     rsv_status st = c->ints.ensure(kIntSlots * sizeof(int));
     if (st == RSV_OK) st = c->partials.ensure(4096 * sizeof(double));
+    if (st == RSV_OK) st = c->target_sums.ensure(target_blocks() * sizeof(double));
     if (st == RSV_OK) st = c->scalars.ensure(64 * sizeof(double));
     if (st != RSV_OK) {
         rsv_destroy(c);

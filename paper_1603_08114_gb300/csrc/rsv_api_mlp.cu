@@ -29,9 +29,8 @@ rsv_status rsv_welford_target(rsv_ctx* c, const double* mean, const double* m2, 
     if (st != RSV_OK) return st;
     if (!mean || !m2 || !target_out) return fail(RSV_EINVAL, "null argument");
     if (T < 1 || count < 2) return fail(RSV_EINVAL, "need T >= 1 and count >= 2");
-    // (the context's partials hold 4096 doubles from its creation on)
     cudaError_t e = counted(c, launch_welford_target, mean, m2, T, count, hbar_out, target_out,
-                            log_scale_out, c->partials.as<double>(),
+                            log_scale_out, c->target_sums.as<double>(),
                             reinterpret_cast<unsigned*>(c->ints.as<int>() + kBatchCounter + 3),
                             (cudaStream_t)stream);
     return e == cudaSuccess ? RSV_OK : cuda_fail(e, "welford target kernel");

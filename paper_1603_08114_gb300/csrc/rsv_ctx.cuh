@@ -77,6 +77,10 @@ struct rsv_ctx {
     rsv::Buf ints;      // int slots
     rsv::Buf scalars;   // double scratch scalars
     rsv::Buf partials;  // per-block partial sums
+    // block sums of rsv_welford_target, of one size from creation on and used by
+    // nothing else: that call may be captured, or run beside a chain of this
+    // context on another stream
+    rsv::Buf target_sums;
     rsv::Buf dbuf0, dbuf1;  // FP64 [T] scratch (proposal h', p')
     rsv::Buf fbuf0, fbuf1;  // (hi, lo) FP32 state double buffer
     rsv::Buf a_f, lr_f;  // mixed-path per-site constants
@@ -87,7 +91,7 @@ struct rsv_ctx {
     rsv::Buf extra;     // other kernels' scratch
     std::vector<rsv::Buf*> all_bufs()
     {
-        return {&ints, &scalars, &partials, &dbuf0, &dbuf1, &fbuf0, &fbuf1, &a_f, &lr_f, &theta_f,
+        return {&ints, &scalars, &partials, &target_sums, &dbuf0, &dbuf1, &fbuf0, &fbuf1, &a_f, &lr_f, &theta_f,
                 &rstats, &gibbs, &batch, &extra, &ser_cur, &ser_cnt, &ser_dh, &ser_acc};
     }
 };

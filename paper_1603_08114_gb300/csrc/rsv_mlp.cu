@@ -992,10 +992,11 @@ __global__ void __launch_bounds__(256) k_feat_write(const double* __restrict__ y
     }
 }
 
+constexpr int kGrid1Max = 152 * 8;
 int grid1(int64_t n)
 {
     int64_t g = (n + 255) / 256;
-    if (g > 152 * 8) g = 152 * 8;
+    if (g > kGrid1Max) g = kGrid1Max;
     return (int)(g < 1 ? 1 : g);
 }
 
@@ -1120,6 +1121,7 @@ cudaError_t launch_welford_target(const double* mean, const double* m2, int64_t 
     return cudaGetLastError();
 }
 
+size_t target_blocks() { return kGrid1Max; }
 int feat_grid(int64_t T) { return grid1(T); }
 
 cudaError_t launch_features(const double* y, const double* lnrv, const double* hbar, int64_t T,

@@ -31,7 +31,8 @@ cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, c
                             float* m_out, cudaStream_t st);
 cudaError_t launch_welford(const float* x, int64_t n, int64_t T, int64_t count, double* mean,
                            double* m2, cudaStream_t st);
-// partials: 1216 doubles (a block's sum each), counter: zero between launches.
+// partials: target_blocks() doubles (a block's sum each), counter: zero between launches.
+size_t target_blocks();
 cudaError_t launch_welford_target(const double* mean, const double* m2, int64_t T, int64_t count,
                                   double* hbar, float* target, float* log_scale, double* partials,
                                   unsigned* counter, cudaStream_t st);
