@@ -862,38 +862,60 @@ __device__ __forceinline__ float const_feature(int f, const ThetaD& th)
 
 // Mean and 1/sd of every feature over the sites, stats = [mean(20), inv_sd(20)]:
 // one pass over the inputs (24 B a site), sums in FP64 of the four site
-// features about their values at the middle site; the nine hbar columns are
-// the same values up to the few at the ends, constants are exact.  (The
-// features were written out, 80 B a site, read back twice for the statistics
-// and once to be standardised in place: 640 us at 2^20 sites, 110 now.)
-constexpr int kFeatSums = 8;
-__global__ void __launch_bounds__(256) k_feat_stats(const double* __restrict__ y,
-                                                    const double* __restrict__ lnrv,
-                                                    const double* __restrict__ hbar, int64_t T,
-                                                    ThetaD th, double* __restrict__ partials,
-                                                    unsigned* __restrict__ counter,
-                                                    float* __restrict__ stats)
+// features about centres near their means, so that the squares keep the
+// accuracy of a second pass: the mean of up to 256 sites spread over the
+// series, which every block takes for itself.  (That mean is within sd
+// sqrt(T / 256) of the mean, which costs the variance at most T / 256 ulp.)  The
+// nine hbar columns are the same values but for the four sites at either end,
+// which some columns leave out: hbar is summed without them and each column
+// adds its own; constants are exact.  (The features were written out, 80 B a
+// site, read back twice for the statistics and once to be standardised in
+// place: 640 us at 2^20 sites, 110 now.)
+constexpr int kFeatSums = 8, kFeatThreads = 256, kWing = 4;
+__global__ void __launch_bounds__(kFeatThreads) k_feat_stats(
+    const double* __restrict__ y, const double* __restrict__ lnrv, const double* __restrict__ hbar,
+    int64_t T, ThetaD th, double* __restrict__ partials, unsigned* __restrict__ counter,
+    float* __restrict__ stats)
 {
-    __shared__ double red[32], tot[kFeatSums];
+    __shared__ double red[32], tot[kFeatSums], s_cf[4], buf[4][kFeatThreads];
     __shared__ u64 s_exp[kExpN];
     __shared__ int s_last;
+    const int tid = threadIdx.x;
     exp_table(s_exp);
     __syncthreads();
-    const int64_t mid = T / 2;
-    const SiteFeat c = site_features(y[mid], lnrv[mid], hbar[mid], s_exp);
-    const float cv[4] = {c.y2, c.lr, c.hb, c.ey};
     double cf[4];  // the centres (any finite value serves)
+    {
+        const int64_t m = T < kFeatThreads ? T : kFeatThreads, t = tid * T / m + T / (2 * m);
+        const bool act = tid < m, in = act && t >= kWing && t < T - kWing;
+        double v[4] = {0.0, 0.0, 0.0, 0.0};
+        if (act) {
+            const SiteFeat q = site_features(y[t], lnrv[t], hbar[t], s_exp);
+            v[0] = q.y2;
+            v[1] = q.lr;
+            v[2] = in ? q.hb : 0.f;
+            v[3] = q.ey;
+        }
+        const int n_in = __syncthreads_count(in);
+        block_sum_many<4, kFeatThreads>(v, buf, tot);
+        if (tid < 4) {
+            const double c = tot[tid] / (tid == 2 ? (double)(n_in > 0 ? n_in : 1) : (double)m);
+            s_cf[tid] = isfinite(c) ? c : 0.0;
+        }
+        __syncthreads();
+    }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) cf[i] = isfinite(cv[i]) ? (double)cv[i] : 0.0;
+    for (int i = 0; i < 4; ++i) cf[i] = s_cf[i];
     double sum[kFeatSums];
 #pragma unroll
     for (int i = 0; i < kFeatSums; ++i) sum[i] = 0.0;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < T;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + tid; t < T;
          t += (int64_t)gridDim.x * blockDim.x) {
         const SiteFeat q = site_features(y[t], lnrv[t], hbar[t], s_exp);
         const float v[4] = {q.y2, q.lr, q.hb, q.ey};
+        const bool in = t >= kWing && t < T - kWing;
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
+            if (i == 2 && !in) continue;
             const double d = f32_to_f64(v[i]) - cf[i];
             sum[2 * i] += d;
             sum[2 * i + 1] = fma(d, d, sum[2 * i + 1]);
@@ -902,12 +924,12 @@ __global__ void __launch_bounds__(256) k_feat_stats(const double* __restrict__ y
 #pragma unroll
     for (int i = 0; i < kFeatSums; ++i) {
         const double b = block_sum(sum[i], red);
-        if (threadIdx.x == 0) partials[(int64_t)blockIdx.x * kFeatSums + i] = b;
+        if (tid == 0) partials[(int64_t)blockIdx.x * kFeatSums + i] = b;
     }
     if (!last_block(counter, &s_last)) return;
     {   // warp i adds sum i over the blocks
-        const int i = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        static_assert(kFeatSums * 32 == 256, "one warp per sum");
+        const int i = tid >> 5, lane = tid & 31;
+        static_assert(kFeatSums * 32 == kFeatThreads, "one warp per sum");
         double v = 0.0;
         for (int b = lane; b < (int)gridDim.x; b += 32)
             v += __ldcg(partials + (int64_t)b * kFeatSums + i);
@@ -915,7 +937,7 @@ __global__ void __launch_bounds__(256) k_feat_stats(const double* __restrict__ y
         if (lane == 0) tot[i] = v;
     }
     __syncthreads();
-    const int f = threadIdx.x;
+    const int f = tid;
     if (f >= NF) return;
     double s1 = 0.0, s2 = 0.0, cen = 0.0;
     if (f == 0 || f == 1 || f == 19) {
@@ -924,15 +946,29 @@ __global__ void __launch_bounds__(256) k_feat_stats(const double* __restrict__ y
         s1 = tot[2 * i];
         s2 = tot[2 * i + 1];
     } else if (f >= 2 && f <= 10) {
-        // column of hbar_{t+k}: the values without the first k (last -k) ones, and as many zeros
-        const int k = f - 6, n = (int)(T < (k < 0 ? -k : k) ? T : (k < 0 ? -k : k));
-        cen = cf[2];
-        s1 = tot[4];
-        s2 = tot[5];
-        for (int j = 0; j < n; ++j) {
-            const double d = (double)(float)hbar[k > 0 ? j : T - 1 - j] - cen;
-            s1 -= d + cen;
-            s2 += cen * cen - d * d;
+        // the column of hbar_{t+k}: sites j = max(k, 0) .. min(T, T + k) - 1, |k| zeros
+        const int64_t k = f - 6, lo = k > 0 ? k : 0, hi = k < 0 ? T + k : T;
+        if (T <= 2 * kWing) {  // no site between the ends: two passes over the column
+            for (int64_t j = lo; j < hi; ++j) s1 += (double)(float)hbar[j];
+            cen = s1 / (double)T;
+            s1 = 0.0;
+            for (int64_t t = 0; t < T; ++t) {
+                const int64_t j = t + k;
+                const double d = (j >= 0 && j < T ? (double)(float)hbar[j] : 0.0) - cen;
+                s2 = fma(d, d, s2);
+            }
+        } else {
+            const double nz = (double)(k < 0 ? -k : k);
+            cen = cf[2];
+            s1 = fma(-nz, cen, tot[4]);
+            s2 = fma(nz * cen, cen, tot[5]);
+            for (int e = 0; e < 2 * kWing; ++e) {
+                const int64_t j = e < kWing ? e : T - 2 * kWing + e;
+                if (j < lo || j >= hi) continue;
+                const double d = (double)(float)hbar[j] - cen;
+                s1 += d;
+                s2 = fma(d, d, s2);
+            }
         }
     } else if (f != EDGE) {
         cen = (double)const_feature(f, th);
@@ -1130,7 +1166,7 @@ cudaError_t launch_features(const double* y, const double* lnrv, const double* h
 {
     // two blocks per SM: a block's FP64 reductions cost as much as a few hundred sites
     const int g = grid1(T);
-    k_feat_stats<<<g < 304 ? g : 304, 256, 0, st>>>(y, lnrv, hbar, T, th, partials, counter, stats);
+    k_feat_stats<<<g < 304 ? g : 304, kFeatThreads, 0, st>>>(y, lnrv, hbar, T, th, partials, counter, stats);
     k_feat_write<<<g, 256, 0, st>>>(y, lnrv, hbar, T, th, stats, F);
     return cudaGetLastError();
 }
