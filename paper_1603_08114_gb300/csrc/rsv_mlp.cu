@@ -877,7 +877,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_feat_stats(
     int64_t T, ThetaD th, double* __restrict__ partials, unsigned* __restrict__ counter,
     float* __restrict__ stats)
 {
-    __shared__ double red[32], tot[kFeatSums], s_cf[4], buf[4][kFeatThreads];
+    __shared__ double red[32], tot[kFeatSums], s_cf[4], s_end[2 * kWing], buf[4][kFeatThreads];
     __shared__ u64 s_exp[kExpN];
     __shared__ int s_last;
     const int tid = threadIdx.x;
@@ -895,6 +895,8 @@ __global__ void __launch_bounds__(kFeatThreads) k_feat_stats(
             v[2] = in ? q.hb : 0.f;
             v[3] = q.ey;
         }
+        if (tid < 2 * kWing && T > 2 * kWing)  // the sites at the ends, for the finish
+            s_end[tid] = (double)(float)hbar[tid < kWing ? tid : T - 2 * kWing + tid];
         const int n_in = __syncthreads_count(in);
         block_sum_many<4, kFeatThreads>(v, buf, tot);
         if (tid < 4) {
@@ -965,7 +967,7 @@ __global__ void __launch_bounds__(kFeatThreads) k_feat_stats(
             for (int e = 0; e < 2 * kWing; ++e) {
                 const int64_t j = e < kWing ? e : T - 2 * kWing + e;
                 if (j < lo || j >= hi) continue;
-                const double d = (double)(float)hbar[j] - cen;
+                const double d = s_end[e] - cen;
                 s1 += d;
                 s2 = fma(d, d, s2);
             }
