@@ -354,7 +354,10 @@ rsv_status rsv_gibbs_theta(rsv_ctx* ctx, const double* h, const double* lnrv, in
  *   {k/4, step, 3, 0}, key {seed, 0}.  batch: multiple of 64.  T < 2^32.
  * rsv_mlp_train: n_steps Adam steps (steps step0 .. step0+n_steps-1, Adam time
  *   step+1) on params with state adam_m, adam_v (FP32 [RSV_MLP_NPARAM], zero
- *   before step 0); loss_out [n_steps] or NULL.
+ *   before step 0); loss_out [n_steps] or NULL.  Several steps run as one
+ *   launch whose blocks wait for one another: on RSV_ETIMEOUT from
+ *   rsv_sync_status() params, the Adam state and loss_out are those of an
+ *   unfinished step, not to be used (check before rsv_mlp_mass is relied on).
  * rsv_mlp_mass: minv_out [T] = 1/m_t and, if m_out != NULL, m_out [T] = m_t,
  *   with m_t clamped to [1/s_u^2, A_t/s_eta^2 + 1/s_u^2 + (y_t^2/2) e^{-hbar_t}]
  *   (the observation precision, a floor of the posterior precision, and the

@@ -237,12 +237,14 @@ rsv_status rsv_sync_status(rsv_ctx* c, void* stream)
 {
     rsv_status st = ctx_begin(c, stream);
     if (st != RSV_OK) return st;
-    cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     int w = 0;
-    e = cudaMemcpy(&w, c->ints.as<int>() + kStatus, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaMemcpyAsync(&w, c->ints.as<int>() + kStatus, sizeof(int),
+                                    cudaMemcpyDeviceToHost, (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "read status");
-    e = cudaMemset(c->ints.as<int>() + kStatus, 0, sizeof(int));
+    e = cudaStreamSynchronize((cudaStream_t)stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
+    if (w == 0) return RSV_OK;
+    e = cudaMemsetAsync(c->ints.as<int>() + kStatus, 0, sizeof(int), (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(e, "clear status");
     if (w & ST_TIMEOUT) return fail(RSV_ETIMEOUT, "a device-side wait ran out of time");
     if (w & ST_NONFINITE) return fail(RSV_ENONFINITE, "a dH was not finite (trajectory rejected)");

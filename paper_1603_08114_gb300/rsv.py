@@ -135,6 +135,9 @@ class Context:
 
     def __init__(self, device: int = 0):
         self.device = device
+        # a non-finite dH found by a check in between (check_timeout), which the
+        # next rsv_sync_status reports
+        self.nonfinite = False
         h = _P()
         _check(lib().rsv_create(ctypes.byref(h), int(device)))
         self.handle = h
@@ -205,10 +208,20 @@ def rsv_sync_status(ctx: Context, allow_nonfinite: bool = False) -> int:
     whose dH was not finite, rejected by the Metropolis test) is returned
     instead of raised."""
     st = lib().rsv_sync_status(ctx.handle, _stream())
+    if st != RSV_ETIMEOUT and ctx.nonfinite:
+        st = RSV_ENONFINITE
+    ctx.nonfinite = False
     if allow_nonfinite and st == RSV_ENONFINITE:
         return st
     _check(st)
     return st
+
+
+def check_timeout(ctx: Context):
+    """Synchronise the current stream and raise RSV_ETIMEOUT if a device-side wait
+    ran out; a non-finite dH stays for the next rsv_sync_status."""
+    if rsv_sync_status(ctx, allow_nonfinite=True) == RSV_ENONFINITE:
+        ctx.nonfinite = True
 
 
 def rsv_action(ctx: Context, h, y, lnrv, th, S_out=None):
