@@ -101,7 +101,10 @@ rsv_status rsv_set_schedule(rsv_ctx* ctx, int threads, int sites_per_thread, int
  * kernel after it).  Every tile stays on its SM for the whole chain; after
  * each trajectory one grid barrier, then every block sums all tiles' records
  * in the same order and takes the same Metropolis decision and theta sweep.
- * The results are bit for bit those of the per-trajectory launches. */
+ * On one tiling (rsv_set_schedule) the results are bit for bit those of the
+ * per-trajectory launches; the automatic tilings of the two differ, and with
+ * them dH by the order of its sums.  Chains with leverage and FP64 chains do not
+ * depend on the switch: they take the tiling of rsv_hmc_trajectory. */
 rsv_status rsv_set_persistent(rsv_ctx* ctx, int enable);
 /* rsv_set_wait_limit: the clock cycles (per SM) a device-side wait of the
  * persistent chain or of rsv_mlp_train may spin before it gives up: it then
@@ -250,8 +253,8 @@ rsv_status rsv_hmc_trajectory(rsv_ctx* ctx, double* h, double* p, const double* 
  *  mass_used_out: device int32 scalar (1 while the mass is in use), or NULL.
  * In RSV_MIXED precision on the model without leverage the whole call runs as
  * one persistent cooperative launch when the plan's tiles can all be resident
- * (see rsv_set_persistent, rsv_chain_schedule); the results equal those of
- * one launch per trajectory bit for bit. */
+ * (see rsv_set_persistent, rsv_chain_schedule); on one tiling the results equal
+ * those of one launch per trajectory bit for bit. */
 rsv_status rsv_hmc_chain(rsv_ctx* ctx, double* h, const double* y, const double* lnrv, int64_t T,
                          double* theta, const float* minv, int n_md, double dtau,
                          rsv_precision prec, uint64_t seed, uint64_t traj0, int64_t n_traj,

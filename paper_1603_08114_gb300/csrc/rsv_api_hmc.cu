@@ -44,11 +44,10 @@ cudaError_t timed_traj(rsv_ctx* c, const TrajArgs& a, const Plan& p, cudaStream_
     return e;
 }
 
-// Single-series plan from the context cache.  chain: the plan of a mixed
-// rsv_hmc_chain call (its own block shape preference; without leverage it can
-// run as one persistent launch).
+// Single-series plan from the context cache.  chain: the block shape by the
+// time model of chains, else that of single trajectories.
 rsv_status single_plan(rsv_ctx* c, int64_t T, int n_md, bool mixed, bool mass, const Plan** out,
-                       bool chain = false)
+                       bool chain)
 {
     for (auto& e : c->plans) {
         if (e.T == T && e.n_md == n_md && e.mixed == mixed && e.mass == mass &&
@@ -77,6 +76,15 @@ rsv_status single_plan(rsv_ctx* c, int64_t T, int n_md, bool mixed, bool mass, c
     c->plans.push_back(e);
     *out = &c->plans.back().plan;
     return RSV_OK;
+}
+
+// Which calls take the time model's shape: chains that may run as one persistent
+// launch, and with leverage, where every trajectory is a launch of its own, every
+// call: a chain's dH is then that of rsv_hmc_trajectory whatever
+// rsv_set_persistent says.
+bool chain_shape(const rsv_ctx* c, rsv_precision prec, bool is_chain)
+{
+    return prec == RSV_MIXED && (c->rho != 0.0 || (is_chain && c->persistent));
 }
 
 // Workspace for a plan: partials per segment, per-series selectors, counters
@@ -377,7 +385,9 @@ rsv_status rsv_hmc_trajectory(rsv_ctx* c, double* h, double* p, const double* y,
     if (!theta_ok(theta)) return fail(RSV_EINVAL, "invalid theta");
     if ((st = check_common(n_md, dtau, prec)) != RSV_OK) return st;
     const Plan* P = nullptr;
-    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, minv != nullptr, &P)) != RSV_OK) return st;
+    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, minv != nullptr, &P,
+                          chain_shape(c, prec, false))) != RSV_OK)
+        return st;
     RunOpts o;
     memset(&o, 0, sizeof(o));
     o.h = h;
@@ -416,8 +426,8 @@ rsv_status rsv_hmc_chain(rsv_ctx* c, double* h, const double* y, const double* l
     if (update_theta && c->rho != 0.0)
         return fail(RSV_EINVAL, "the theta update is for the model without leverage (rho = 0)");
     const Plan* P = nullptr;
-    const bool chain = prec == RSV_MIXED && c->persistent;  // a chain's block shape
-    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, minv != nullptr, &P, chain)) != RSV_OK)
+    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, minv != nullptr, &P,
+                          chain_shape(c, prec, true))) != RSV_OK)
         return st;
     RunOpts o;
     memset(&o, 0, sizeof(o));
@@ -450,12 +460,12 @@ rsv_status rsv_chain_schedule(rsv_ctx* c, int64_t T, int n_md, rsv_precision pre
     if (st != RSV_OK) return st;
     if (T < 1) return fail(RSV_EINVAL, "T must be >= 1 (got %lld)", (long long)T);
     if ((st = check_common(n_md, 1.0, prec)) != RSV_OK) return st;
-    const bool chain = prec == RSV_MIXED && c->persistent;
     const Plan* P = nullptr;
-    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, with_mass != 0, &P, chain)) != RSV_OK)
+    if ((st = single_plan(c, T, n_md, prec == RSV_MIXED, with_mass != 0, &P,
+                          chain_shape(c, prec, true))) != RSV_OK)
         return st;
     bool fits = false;
-    if (chain && c->rho == 0.0) {
+    if (prec == RSV_MIXED && c->persistent && c->rho == 0.0) {
         cudaError_t e = chain_fits(*P, c->num_sms, &fits);
         if (e != cudaSuccess) return cuda_fail(e, "chain occupancy");
     }

@@ -66,7 +66,14 @@ bool valid_j(bool mixed, int j)
 // (74 of 128 x 4) against 33.0, T = 700000, 90 steps 66 (142 of 640 x 8)
 // against 72 (256 x 20); at 2^20 sites only the windows of 384 x 20 fit in one
 // round of 12 warps (87 us with 78 steps and a mass; 448 x 16: 90, 608 x 12:
-// 94).  With leverage a step takes about 1.4 times as long.
+// 94).
+//
+// Mixed with leverage (a launch per trajectory; T = 700 .. 2^22, 8 .. 100 steps,
+// with and without a mass): a step takes about 1.4 times as long (1.3 with runs
+// of 12), and the energies at both ends, per site here, 0.75 j more.  2^20
+// sites: 8 steps 608 x 12 52.6 us against 57.7 (352 x 20), 100 steps 139.3 against
+// 136.0 (384 x 20); over 72 sizes the shape taken is 1.0 % off the fastest on
+// average (1.9 % without the 0.75 j, which took 352 x 20 at 8 steps).
 double round_cost(bool mixed, bool lev, int j, double warps, double n_force)
 {
     if (!mixed)
@@ -80,7 +87,8 @@ double round_cost(bool mixed, bool lev, int j, double warps, double n_force)
         case 16: step = 0.305 + 0.045 * more, fixed = 19.9 + 0.7 * warps; break;
         default: step = 0.36 + 0.038 * more, fixed = 19.1 + 0.9 * warps; break;
     }
-    return fixed + n_force * step * (lev ? 1.4 : 1.0);
+    if (lev) return fixed + 0.75 * j + n_force * step * (j == 12 ? 1.3 : 1.4);
+    return fixed + n_force * step;
 }
 
 // Bins that whole series of cnt[w] x w warps need at NW warps a bin, larger
@@ -208,7 +216,8 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                                round_cost(false, lev, js[ji], (double)per * (t / 32), (double)(K - 1)) *
                                (1.0 + 1e-6 * b);
                     } else if (chain) {
-                        // one block per SM: a round more is a launch more
+                        // one block per SM; a round more of a chain without
+                        // leverage is a launch more
                         const int64_t w = (b + num_sms - 1) / num_sms;
                         cost = (double)w * (round_cost(true, lev, js[ji], t / 32, (double)(K - 1)) +
                                             (w > 1 ? 6.0 : 0.0)) + 0.005 * b;
