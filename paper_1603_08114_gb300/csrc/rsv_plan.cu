@@ -66,7 +66,10 @@ bool valid_j(bool mixed, int j)
 // (74 of 128 x 4) against 33.0, T = 700000, 90 steps 66 (142 of 640 x 8)
 // against 72 (256 x 20); at 2^20 sites only the windows of 384 x 20 fit in one
 // round of 12 warps (87 us with 78 steps and a mass; 448 x 16: 90, 608 x 12:
-// 94).
+// 94).  Below four warps the draws, the sweep and the decision wait for one
+// another: T = 2000, 6 force evaluations 13.5 us (5 blocks of 128 x 4) against 19.4
+// (19 of 32 x 4) and 17.1 (one of 512 x 4).  T = 500 .. 2^20, 2 .. 60 evaluations:
+// the shape taken is 0.8 % off the fastest on average (17 % without that term).
 //
 // Mixed with leverage (a launch per trajectory; T = 700 .. 2^22, 8 .. 100 steps,
 // with and without a mass): a step takes about 1.4 times as long (1.3 with runs
@@ -79,9 +82,12 @@ double round_cost(bool mixed, bool lev, int j, double warps, double n_force)
     if (!mixed)
         return 16.0 + 3.0 * j + n_force * std::max(0.30 + 0.36 * j, 0.50 + 0.0625 * j * warps);
     const double more = std::max(0.0, warps - 4.0);
+    // few warps take the serial phases one after another
+    const double alone = lev ? (warps < 2.0 ? 1.5 : 0.0)
+                         : warps < 2.0 ? 4.0 : warps < 3.0 ? 1.5 : warps < 4.0 ? 0.6 : 0.0;
     double step, fixed;
     switch (j) {
-        case 4: step = 0.147 + 0.0119 * more, fixed = 13.3 + 0.22 * warps; break;
+        case 4: step = 0.147 + 0.0119 * more, fixed = 13.3 + 0.22 * warps + alone; break;
         case 8: step = 0.21 + 0.0195 * more, fixed = 16.0 + 0.22 * warps; break;
         case 12: step = 0.32 + 0.031 * more, fixed = 20.0 + 0.55 * warps; break;
         case 16: step = 0.305 + 0.045 * more, fixed = 19.9 + 0.7 * warps; break;
