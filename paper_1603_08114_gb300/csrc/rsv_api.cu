@@ -125,7 +125,6 @@ rsv_status rsv_create(rsv_ctx** out, int device)
     rsv_status st = c->ints.ensure(kIntSlots * sizeof(int));
     if (st == RSV_OK) st = c->partials.ensure(4096 * sizeof(double));
     if (st == RSV_OK) st = c->target_sums.ensure(target_blocks() * sizeof(double));
-    if (st == RSV_OK) st = c->scalars.ensure(64 * sizeof(double));
     if (st != RSV_OK) {
         rsv_destroy(c);
         return st;

@@ -35,7 +35,6 @@ enum IntSlot : int {
     kBatchCounter = 16,  // [..] per-call counters of other kernels
     kIntSlots = 64
 };
-enum ScalSlot : int { kScalDH = 0 };
 
 }  // namespace rsv
 
@@ -75,7 +74,6 @@ struct rsv_ctx {
     std::vector<cudaEvent_t> ev;  // pairs (start, stop)
     size_t ev_used = 0;
     rsv::Buf ints;      // int slots
-    rsv::Buf scalars;   // double scratch scalars
     rsv::Buf partials;  // per-block partial sums
     // block sums of rsv_welford_target, of one size from creation on and used by
     // nothing else: that call may be captured, or run beside a chain of this
@@ -91,7 +89,7 @@ struct rsv_ctx {
     rsv::Buf extra;     // other kernels' scratch
     std::vector<rsv::Buf*> all_bufs()
     {
-        return {&ints, &scalars, &partials, &target_sums, &dbuf0, &dbuf1, &fbuf0, &fbuf1, &a_f, &lr_f, &theta_f,
+        return {&ints, &partials, &target_sums, &dbuf0, &dbuf1, &fbuf0, &fbuf1, &a_f, &lr_f, &theta_f,
                 &rstats, &gibbs, &batch, &extra, &ser_cur, &ser_cnt, &ser_dh, &ser_acc};
     }
 };
