@@ -1,9 +1,10 @@
 """Autotuner for the block shape of the trajectory kernels.
 
-A candidate is (threads per block, sites per thread); the tile of a series cut
-into tiles is the largest the window allows.  Each candidate's plan is built
-(`rsv_set_schedule` + `rsv_plan_create`) and one trajectory of the workload is
-timed with CUDA events; the fastest wins.  Results are cached in a JSON file
+The first candidate is the plan that `rsv_plan_create` makes by itself, so that a
+tuned plan is no slower; the others are (threads per block, sites per thread),
+the tile of a series cut into tiles the largest the window allows
+(`rsv_set_schedule` + `rsv_plan_create`).  One trajectory of the workload is timed
+on each with CUDA events; the fastest wins.  Results are cached in a JSON file
 keyed by GPU name, precision, n_md, mass and a size bucket of the workload, so
 later runs skip the search.  Results never change the numbers a plan computes,
 only its speed.
@@ -19,15 +20,16 @@ import torch
 
 from . import rsv
 
-# bumped whenever the trajectory kernels change, so cached choices are redone
-KERNEL_REV = 16
+# bumped whenever the trajectory kernels or the candidates change, so cached
+# choices are redone
+KERNEL_REV = 17
 
 CANDIDATES = {
     "mixed": ([(nt, 20) for nt in (128, 192, 256, 320, 384)]
               + [(nt, 16) for nt in (128, 256, 384, 512)]
               + [(nt, 12) for nt in (192, 320, 448, 640)]
               + [(nt, 8) for nt in (256, 384, 512, 768)]),
-    "fp64": [(nt, j) for j in (8, 16, 28) for nt in (64, 128, 192, 256)],
+    "fp64": [(nt, j) for j in (1, 2, 4, 8, 16, 28) for nt in (64, 128, 192, 256)],
 }
 
 
@@ -59,27 +61,31 @@ def tune_plan(ctx: rsv.Context, offsets, n_md: int, prec: str, y, lnrv, theta_de
         except (OSError, ValueError):
             cache = {}
     K = n_md + 1
-    if use_cache and key in cache:
-        nt, j = cache[key]["threads"], cache[key]["sites_per_thread"]
-        rsv.rsv_set_schedule(ctx, nt, j, nt * j - 2 * K - 3)
+
+    def make(shape):
+        """The plan on a fixed (threads, sites per thread), or None: the automatic one."""
+        nt, j = shape or (0, 0)
+        rsv.rsv_set_schedule(ctx, nt, j, nt * j - 2 * K - 3 if shape else 0)
         try:
-            plan = rsv.Plan(ctx, offsets, n_md, prec, with_mass=minv is not None)
+            return rsv.Plan(ctx, offsets, n_md, prec, with_mass=minv is not None)
         finally:
             rsv.rsv_set_schedule(ctx)
-        return plan, dict(cache[key], cached=True)
+
+    if use_cache and key in cache:
+        e = cache[key]
+        plan = make(None if e["automatic"] else (e["threads"], e["sites_per_thread"]))
+        return plan, dict(e, cached=True)
     results = []
     h = torch.empty_like(h_init)
-    for nt, j in CANDIDATES["mixed" if prec == "mixed" else "fp64"]:
-        tile = nt * j - 2 * K - 3
-        if tile < 1:
+    for shape in [None] + CANDIDATES["mixed" if prec == "mixed" else "fp64"]:
+        if shape is not None and shape[0] * shape[1] - 2 * K - 3 < 1:
             continue
         try:
-            rsv.rsv_set_schedule(ctx, nt, j, tile)
-            plan = rsv.Plan(ctx, offsets, n_md, prec, with_mass=minv is not None)
+            plan = make(shape)
         except rsv.RSVError:
+            if shape is None:
+                raise
             continue
-        finally:
-            rsv.rsv_set_schedule(ctx)
         times = []
         for r in range(reps + 1):
             h.copy_(h_init)
@@ -91,21 +97,18 @@ def tune_plan(ctx: rsv.Context, offsets, n_md: int, prec: str, y, lnrv, theta_de
             b.synchronize()
             if r:
                 times.append(a.elapsed_time(b))
-        results.append((min(times), nt, j, plan.info()))
+        results.append((min(times), shape, plan.info()))
         plan.close()
     results.sort(key=lambda r: r[0])
-    best_ms, nt, j, info = results[0]
-    entry = {"threads": nt, "sites_per_thread": j, "ms": best_ms, "info": info,
-             "candidates": [(round(t, 4), a, b) for t, a, b, _ in results]}
+    best_ms, shape, info = results[0]
+    entry = {"automatic": shape is None, "threads": info["threads"],
+             "sites_per_thread": info["sites_per_thread"], "ms": best_ms, "info": info,
+             "candidates": [(round(t, 4), i["threads"], i["sites_per_thread"], s is None)
+                            for t, s, i in results]}
     cache[key] = entry
     try:
         with open(path, "w") as f:
             json.dump(cache, f, indent=1)
     except OSError:
         pass
-    rsv.rsv_set_schedule(ctx, nt, j, nt * j - 2 * K - 3)
-    try:
-        plan = rsv.Plan(ctx, offsets, n_md, prec, with_mass=minv is not None)
-    finally:
-        rsv.rsv_set_schedule(ctx)
-    return plan, dict(entry, cached=False)
+    return make(shape), dict(entry, cached=False)
