@@ -91,8 +91,9 @@ rsv_status rsv_sync_status(rsv_ctx* ctx, void* stream);
  * into tiles (tile + 2 (n_md + 1) + 3 <= threads * sites_per_thread, else the
  * call that uses it fails with RSV_EINVAL).  A single series no longer than
  * `tile` is kept whole (it then needs only T <= threads * sites_per_thread).
- * All zero restores the automatic plan.  Results depend on the tiling only
- * through rounding (the order of the sums). */
+ * All zero restores the automatic plan.  FP64 results do not depend on the
+ * tiling (dH is summed free of order), mixed ones only through rounding (the
+ * order of the sums). */
 rsv_status rsv_set_schedule(rsv_ctx* ctx, int threads, int sites_per_thread, int64_t tile);
 /* rsv_set_persistent: 1 (the default) runs an rsv_hmc_chain call in RSV_MIXED
  * precision on the model without leverage as ONE persistent cooperative
@@ -292,7 +293,8 @@ rsv_status rsv_plan_info(const rsv_plan* plan, int* threads, int* sites_per_thre
  *  minv     packed FP32 inverse masses or NULL (the plan must match).
  *  log_u    device FP64 [n_series] or NULL (draw); non-NULL only with n_traj = 1.
  *  dH_out, accept_out: device [n_traj][n_series] FP64 / int32, or NULL.
- * With RSV_MIXED the state of a series is carried as a (hi, lo) FP32 pair
+ * On automatic plans a series' results are the same bits whatever it is packed
+ * with (in RSV_MIXED: two series or more).  With RSV_MIXED the state of a series is carried as a (hi, lo) FP32 pair
  * between trajectories (about 48 significant bits); with n_traj = 1 the h of a
  * rejected series is left bit-for-bit unchanged. */
 rsv_status rsv_hmc_batched(rsv_ctx* ctx, rsv_plan* plan, double* h, double* p, const double* y,

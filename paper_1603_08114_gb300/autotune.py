@@ -22,7 +22,7 @@ from . import rsv
 
 # bumped whenever the trajectory kernels or the candidates change, so cached
 # choices are redone
-KERNEL_REV = 17
+KERNEL_REV = 18
 
 CANDIDATES = {
     "mixed": ([(nt, 20) for nt in (128, 192, 256, 320, 384)]

@@ -372,6 +372,60 @@ __device__ __forceinline__ double block_sum(double v, double* red)
     return s;
 }
 
+// A sum of FP64 terms that does not depend on their order, so that a series'
+// dH is the same bits whatever block shape or tiles its sites are spread over:
+// each term cut to a multiple of 2^-64 (its own rounding is coarser from 2^-11 on)
+// and added as a 128-bit integer.  Terms of 2^28 or more, infinities and NaN go
+// to an FP64 sum beside it (|S| < 2^63 for 2^35 terms below that).
+struct FixSum {
+    unsigned long long lo;
+    long long hi;
+    double big;
+};
+__device__ __forceinline__ void fix_merge(FixSum& s, unsigned long long lo, long long hi, double big)
+{
+    s.lo += lo;
+    s.hi += hi + (long long)(s.lo < lo);
+    s.big += big;
+}
+__device__ __forceinline__ void fix_add(FixSum& s, double v)
+{
+    const unsigned h = (unsigned)__double2hiint(v), E = (h >> 20) & 0x7ffu;
+    if (E >= 1051u) {
+        s.big += v;
+        return;
+    }
+    const unsigned long long M = ((unsigned long long)((h & 0xfffffu) | (E ? 0x100000u : 0u)) << 32) |
+                                 (unsigned)__double2loint(v);
+    const int sh = (int)E - 1011;  // |v| 2^64 = M 2^sh, sh < 40
+    unsigned long long lo = sh >= 0 ? M << sh : sh > -64 ? M >> -sh : 0ull;
+    long long hi = sh > 0 ? (long long)(M >> (64 - sh)) : 0ll;
+    if ((int)h < 0) {
+        lo = 0ull - lo;
+        hi = ~hi + (long long)(lo == 0ull);
+    }
+    s.lo += lo;
+    s.hi += hi + (long long)(s.lo < lo);
+}
+__device__ __forceinline__ FixSum fix_warp_sum(FixSum s)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, s.lo, o);
+        const long long hi = __shfl_xor_sync(0xffffffffu, s.hi, o);
+        fix_merge(s, lo, hi, __shfl_xor_sync(0xffffffffu, s.big, o));
+    }
+    return s;
+}
+__device__ __forceinline__ double fix_to_double(const FixSum& s)
+{
+    const bool neg = s.hi < 0;
+    const unsigned long long lo = neg ? 0ull - s.lo : s.lo;
+    const long long hi = neg ? ~s.hi + (long long)(lo == 0ull) : s.hi;
+    const double d = fma((double)lo, 0x1p-64, (double)hi);
+    return (neg ? -d : d) + s.big;
+}
+
 // Block sums of N values (blockDim.x = NT threads, NT / 32 >= N warps): warp i
 // adds value i over the threads, lane l those of l, l + 32, ... in order, then
 // a butterfly (a butterfly per warp and value first would take five of the FP64

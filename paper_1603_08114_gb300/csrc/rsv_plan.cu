@@ -257,8 +257,9 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
         // series' double-float sums are taken in the same order whatever it
         // is packed with; smaller blocks spread few short series over the SMs
         // (10 series of 300 .. 1000 sites, 40 steps: 64 x 20 in 7 blocks 54 us a
-        // trajectory, 384 x 20 in 2 78).  FP64 takes any run (64 series of 300
-        // .. 2000: 192 x 2 120 us a trajectory, 256 x 28 702).
+        // trajectory, 384 x 20 in 2 78).  FP64, whose sums have no order, takes
+        // any run (64 series of 300 .. 2000: 192 x 2 120 us a trajectory, 256 x 28
+        // 702).
         double best = 1e300;
         const int big_j = mixed ? 20 : 28, big_t = ntmax(mixed, mass, big_j);
         if ((int64_t)big_t * big_j - 2 * K - 3 < 1) {

@@ -61,7 +61,8 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_wseg[NWMAX], s_wacc[NWMAX], s_flag;
-    __shared__ double s_wpart[NWMAX], s_red[32], s_edge[4 * NWMAX], s_split;
+    __shared__ double s_edge[4 * NWMAX];
+    __shared__ FixSum s_wpart[NWMAX], s_split;
     __shared__ u64 s_e2[kExpN];  // the table of exp_neg
     const int NT = blockDim.x, W = NT * J, nw = NT >> 5, tid = threadIdx.x;
     exp_table(s_e2);  // read after load_bin's barriers
@@ -142,10 +143,13 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
         // leverage: y e^{-mu/2} of the left neighbour site (none at a window start)
         const double yL = (LEV && !v.first) ? s_a[(J - 1) * NT + tid - 1] : 0.0;
 
-        // H restricted to this thread's owned sites (x coordinates; the
-        // constant mu/2 per site cancels in dH).
+        // dH restricted to this thread's owned sites: -H of each at the start
+        // and +H at the end (x coordinates; the constant mu/2 per site cancels),
+        // every term the same operations whatever the shape, their sum free
+        // of the order they are taken in.
         int par = 0;
-        auto owned_energy = [&](double& acc) {
+        auto owned_energy = [&](double sign) {
+            FixSum dE{0ull, 0ll, 0.0};
             double xL, xR;
             exchange(x[0], x[J - 1], xL, xR, s_edge + par * 2 * nw, nw);
             par ^= 1;
@@ -165,16 +169,20 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
                     if (j == la) e = 0.0;
                     const double cp = (A.lnrv[off + s] - th.xi) - mu;
                     const double r = cp - x[j];
-                    double val = 0.5 * x[j] + ey + 0.5 * iu * r * r + 0.5 * ib * e * e;
-                    if (s == 0) val += 0.5 * ie * st0 * x[j] * x[j];
+                    double val = fma(0.5 * iu * r, r, fma(0.5, x[j], ey));
+                    val = fma(0.5 * ib * e, e, val);
+                    if (s == 0) val = fma(0.5 * ie * st0 * x[j], x[j], val);
                     const double mi = MASS ? s_mi[j * NT + tid] : 1.0;
-                    val += 0.5 * mi * p[j] * p[j];
-                    acc += val;
+                    val = fma(0.5 * mi * p[j], p[j], val);
+                    fix_add(dE, sign * val);
                 }
             }
+            return fix_warp_sum(dE);
         };
-        double E0 = 0.0, E1 = 0.0;
-        owned_energy(E0);
+        {   // (kept in shared memory through the steps)
+            const FixSum e0 = owned_energy(-1.0);
+            if ((tid & 31) == 0) s_wpart[tid >> 5] = e0;
+        }
 
         // The scheme (drift a_0 dtau, then {kick b_k dtau; drift a_{k+1}
         // dtau} per step; the leapfrog eqs. (6)-(8) are drift dtau/2, kick
@@ -224,10 +232,8 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
                 }
             }
         }
-        owned_energy(E1);
-
-        const double part = warp_sum(E1 - E0);
-        if ((tid & 31) == 0) s_wpart[tid >> 5] = part;
+        const FixSum e1 = owned_energy(1.0);
+        if ((tid & 31) == 0) fix_merge(s_wpart[tid >> 5], e1.lo, e1.hi, e1.big);
         __syncthreads();
         segment_decisions(A, v, s_wpart, s_wacc, &s_split);
         __syncthreads();
@@ -240,7 +246,7 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
                 if (A.p_out) A.p_out[off + s] = p[j];
             }
         }
-        if (v.g.split) finish_split(A, v, s_split, s_red, &s_flag);
+        if (v.g.split) finish_split(A, v, s_split, s_wpart, &s_flag);
     }
 }
 

@@ -182,12 +182,18 @@ __device__ int decide(const TrajArgs& A, int series, double dH, int cur, bool fl
 }
 
 // The last tile of a split series to arrive sums the partials of all its
-// tiles in tile order and decides.  Called by the whole block.
-__device__ void finish_split(const TrajArgs& A, const View& v, double part, double* red,
+// tiles (kFixWords doubles each) and decides.  Called by the whole block.
+constexpr int kFixWords = 3;
+__device__ void finish_split(const TrajArgs& A, const View& v, const FixSum& part, FixSum* red,
                              int* s_flag)
 {
+    static_assert(kFixWords <= kPartialWords && sizeof(FixSum) == kFixWords * sizeof(double), "room");
+    unsigned long long* pw = reinterpret_cast<unsigned long long*>(A.partials);
     if (threadIdx.x == 0) {
-        A.partials[v.sid] = part;
+        unsigned long long* w = pw + (int64_t)v.sid * kFixWords;
+        w[0] = part.lo;
+        w[1] = (unsigned long long)part.hi;
+        w[2] = (unsigned long long)__double_as_longlong(part.big);
         __threadfence();
         const unsigned prev = atomicAdd(A.ser_cnt + v.g.series, 1u);
         *s_flag = (prev == (unsigned)v.si.nseg - 1u);
@@ -197,27 +203,34 @@ __device__ void finish_split(const TrajArgs& A, const View& v, double part, doub
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double s = 0.0;
-    for (int i = threadIdx.x; i < v.si.nseg; i += blockDim.x) s += __ldcg(A.partials + v.si.seg0 + i);
-    const double dH = block_sum(s, red);
+    FixSum s{0ull, 0ll, 0.0};
+    for (int i = threadIdx.x; i < v.si.nseg; i += blockDim.x) {
+        const unsigned long long* w = pw + (int64_t)(v.si.seg0 + i) * kFixWords;
+        fix_merge(s, __ldcg(w), (long long)__ldcg(w + 1), __longlong_as_double((long long)__ldcg(w + 2)));
+    }
+    s = fix_warp_sum(s);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+    __syncthreads();
     if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) fix_merge(s, red[w].lo, red[w].hi, red[w].big);
         A.ser_cnt[v.g.series] = 0u;
-        decide(A, v.g.series, dH, v.cur, true);
+        decide(A, v.g.series, fix_to_double(s), v.cur, true);
         __threadfence();
     }
 }
 
-// Sum the per-warp parts of each segment (in warp order) and decide whole
-// series; split bins return their part in *split_part.
+// Sum the per-warp parts of each segment and decide whole series; split bins
+// return their part in *split_part.
 __device__ __forceinline__ void segment_decisions(const TrajArgs& A, const View& v,
-                                                  const double* s_wpart, int* s_wacc,
-                                                  double* split_part)
+                                                  const FixSum* s_wpart, int* s_wacc,
+                                                  FixSum* split_part)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (v.sid >= 0 && warp == v.g.warp0 && lane == 0) {
-        double d = 0.0;
-        for (int w = v.g.warp0; w < v.g.warp0 + v.g.nwarp; ++w) d += s_wpart[w];
-        if (!v.g.split) s_wacc[v.g.warp0] = decide(A, v.g.series, d, v.cur, false);
+        FixSum d = s_wpart[warp];
+        for (int w = warp + 1; w < warp + v.g.nwarp; ++w)
+            fix_merge(d, s_wpart[w].lo, s_wpart[w].hi, s_wpart[w].big);
+        if (!v.g.split) s_wacc[warp] = decide(A, v.g.series, fix_to_double(d), v.cur, false);
         else *split_part = d;
     }
 }
