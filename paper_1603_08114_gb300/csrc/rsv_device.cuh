@@ -247,12 +247,13 @@ __device__ __forceinline__ ff ff_exp(ff t, const float2* tab)
 //   e^a = 2^(k div 1024) T (1 + p),  T = 2^((k mod 1024)/1024) to 63 bits,
 //   p = r + r^2/2 + r^3 (1/6 + r/24)   (remainder r^5/120 < 2^-59),
 // the product rounded once, to nearest, into the result's mantissa: within
-// 0.61 ulp of e^a (0.51 away from x = 0; the truncation of a to 2^-56 is the
-// excess), against ~1.1 ulp of the form on FP64 instructions with a 64-entry
-// table that it replaced.  About 55 integer instructions and no FP64 ones, where
-// that form took 10 of the 18 FP64 instructions of a leapfrog step's site.
-// |x| >= 128, NaN, and the one or two arguments in a million whose floor or
-// last carry is ambiguous take CUDA's exp.
+// 0.65 ulp of e^a (the rounding 0.5, the truncation of a to 2^-56 up to 0.125 just
+// below a power of two, the series' remainder 0.016, the truncations of p and T
+// 0.004; largest seen 0.622, 0.51 away from x = 0), against ~1.1 ulp of the form on
+// FP64 instructions with a 64-entry table that it replaced.  About 55 integer
+// instructions and no FP64 ones, where that form took 10 of the 18 FP64
+// instructions of a leapfrog step's site.  |x| >= 128, NaN, and the few arguments
+// in a million whose floor or last carry is ambiguous take CUDA's exp.
 // The table is the products of two 32-entry ones, 2^(i/32) and 2^(j/1024) in
 // units of 2^-63 (rounded from 60 decimal digits).
 // ---------------------------------------------------------------------------
