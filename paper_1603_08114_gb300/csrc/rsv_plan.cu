@@ -97,6 +97,28 @@ double round_cost(bool mixed, bool lev, int j, double warps, double n_force)
     return fixed + n_force * step;
 }
 
+// Time in us of a trajectory of a mixed batch: `bins` bins on blocks of W warps of
+// 20 sites per thread, `bps` blocks to an SM, in rounds of all the blocks that fit
+// and a last one of what is left, as fitted to sweeps of every block size (20 ..
+// 6000 series of 10 .. 7600 sites, 4 .. 50 steps).  k blocks on an SM put k ceil(W /
+// 4) warps on its fullest scheduler, which paces a step; blocks beside one another
+// hide each other's serial phases.  4000 series of 300 .. 640, 50 steps: 128 x 20
+// 142 us, 384 x 20 196, 32 x 20 217 (many one-warp blocks, each in a phase of its
+// own, are slow: blocks below four warps only where every SM has one).  The shape
+// taken is 0.8 % off the fastest on average and 1.4 % with leverage, whose blocks
+// hide less, and at most 1.4 % slower than 384 x 20 (by the model of one block's
+// warps 9 % and 13 % off, and up to 53 % slower than 384 x 20).
+double batch_cost(bool lev, int W, int64_t bins, int64_t bps, int num_sms, double n_force)
+{
+    auto round = [&](int64_t k) {
+        const double s = (double)(k * ((W + 3) / 4)), more = (double)(k - 1);
+        return lev ? 26.7 + 2.4 * s - 0.5 * more + n_force * (0.273 + 0.232 * s + 0.05 * more)
+                   : 19.6 + 2.7 * s - 2.3 * more + n_force * (0.202 + 0.174 * s - 0.109 * more);
+    };
+    const int64_t full = bins / (bps * num_sms), rest = bins % (bps * num_sms);
+    return full * round(bps) + (rest ? round((rest + num_sms - 1) / num_sms) : 0.0);
+}
+
 // Bins that whole series of cnt[w] x w warps need at NW warps a bin, larger
 // ones first, each into the fullest bin with room (an estimate of the packing
 // below, which takes the first such bin).
@@ -295,9 +317,12 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
                 const int bps = blocks_per_sm(mixed, mass, lev, js[ji], t, sm);
                 if (bps < 1) continue;
                 const int64_t per = std::min<int64_t>(bps, (b + num_sms - 1) / num_sms);
+                if (mixed && t < 128 && b > num_sms) continue;
                 const double cost =
-                    (double)((b + per * num_sms - 1) / (per * num_sms)) *
-                    (round_cost(mixed, lev, js[ji], (double)per * (t / 32), (double)(K - 1)) + 6.0);
+                    mixed ? batch_cost(lev, t / 32, b, bps, num_sms, (double)(K - 1))
+                          : (double)((b + per * num_sms - 1) / (per * num_sms)) *
+                                (round_cost(false, lev, js[ji], (double)per * (t / 32),
+                                            (double)(K - 1)) + 6.0);
                 if (cost < best) {
                     best = cost;
                     nt = t;
