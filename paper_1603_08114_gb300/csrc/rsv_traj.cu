@@ -38,6 +38,7 @@
 //   B = 1 / (s_eta^2 (1 - rho^2)),
 // and the y-term (y^2/2) e^{-h} = eps^2 / 2; the stationary term of h_1 is
 // unchanged.
+#include <algorithm>
 #include <array>
 #include <cmath>
 #include <map>
@@ -330,10 +331,12 @@ __device__ __forceinline__ int series_of(const SerInfo* ser, int n, int64_t t)
 }
 
 // The current state back into h: run blockIdx.x of `run` sites of a single
-// series (segs NULL), or the owned sites of segment blockIdx.x, whose series it
-// knows (a search for the series of every packed site was half of the 161 us
-// for 17.7 M sites of 4096 series; the other half FP64 conversions, now one
-// FP64 addition a site: 57 us).
+// series (segs NULL), or part blockIdx.y of gridDim.y of the owned sites of
+// segment blockIdx.x, whose series it knows (a search for the series of every
+// packed site was half of the 161 us for 17.7 M sites of 4096 series; the other
+// half FP64 conversions, now one FP64 addition a site: 57 us).  Few segments are
+// cut in parts, so that a few long series do not wait for a block each (five
+// segments of 7677 sites, cold: 19 us in one part each, 4 in thirty).
 __global__ void __launch_bounds__(256) k_finalize(
     const Seg* __restrict__ segs, const SerInfo* __restrict__ ser, int64_t total, int run,
     const int* __restrict__ cur, const int* __restrict__ acc, const double* __restrict__ h1d,
@@ -344,8 +347,9 @@ __global__ void __launch_bounds__(256) k_finalize(
     if (segs) {
         const Seg g = segs[blockIdx.x];
         s = g.series;
-        lo = ser[s].off + g.lo;
-        hi = ser[s].off + g.hi;
+        const int64_t part = (g.hi - g.lo + gridDim.y - 1) / gridDim.y;
+        lo = ser[s].off + g.lo + blockIdx.y * part;
+        hi = ser[s].off + (g.lo + (blockIdx.y + 1) * part < g.hi ? g.lo + (blockIdx.y + 1) * part : g.hi);
     }
     const int c = cur ? cur[s] : 0;
     if (h0f ? acc && acc[s] == 0 : c == 0) return;
@@ -698,8 +702,11 @@ cudaError_t launch_finalize(const Plan& p, const int* cur, const int* acc, const
     const bool by_seg = p.nseries > 1;
     const int64_t g = by_seg ? p.nsegs : (p.total + run - 1) / run;
     if (g > 0x7fffffff) return cudaErrorInvalidValue;
-    k_finalize<<<(unsigned)g, 256, 0, st>>>(by_seg ? p.d_segs : nullptr, p.d_ser, p.total, run, cur,
-                                            acc, h1d, h0f, h1f, h);
+    // parts down to a site per thread while the segments are fewer than four blocks per SM
+    const int64_t most = ((int64_t)p.nt * p.j + 255) / 256, want = 152 * 4 / g;
+    const int parts = by_seg ? (int)std::max<int64_t>(1, std::min(most, want)) : 1;
+    k_finalize<<<dim3((unsigned)g, parts), 256, 0, st>>>(by_seg ? p.d_segs : nullptr, p.d_ser,
+                                                         p.total, run, cur, acc, h1d, h0f, h1f, h);
     return cudaGetLastError();
 }
 cudaError_t launch_snapshot(const Plan& p, const int* cur, const double* h0d, const double* h1d,
