@@ -403,24 +403,25 @@ bool make_plan(const int64_t* off, int n, int n_md, int integrator, double lambd
         if (!segs[i].split) whole.push_back(i);
     std::stable_sort(whole.begin(), whole.end(),
                      [&](int a, int b) { return segs[a].nwarp > segs[b].nwarp; });
+    // each into the first bin with room: the bins before k have none for the
+    // present size, and never will (rooms only shrink), so the search goes on from k
     std::vector<std::vector<int>> bins;
     std::vector<int> room;
+    int k = 0, size = 0;
     for (int id : whole) {
         const int need = segs[id].nwarp;
-        int b = -1;
-        for (int k = 0; k < (int)bins.size(); ++k)
-            if (room[k] >= need) {
-                b = k;
-                break;
-            }
-        if (b < 0) {
+        if (need != size) {
+            size = need;
+            k = 0;
+        }
+        while (k < (int)bins.size() && room[k] < need) ++k;
+        if (k == (int)bins.size()) {
             bins.emplace_back();
             room.push_back(NW);
-            b = (int)bins.size() - 1;
         }
-        segs[id].warp0 = NW - room[b];
-        room[b] -= need;
-        bins[b].push_back(id);
+        segs[id].warp0 = NW - room[k];
+        room[k] -= need;
+        bins[k].push_back(id);
     }
     for (auto& b : bins) {
         for (int id : b) bin_seg.push_back(id);
