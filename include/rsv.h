@@ -362,13 +362,16 @@ rsv_status rsv_gibbs_theta(rsv_ctx* ctx, const double* h, const double* lnrv, in
  *   before step 0); loss_out [n_steps] or NULL.  Several steps run as one
  *   launch whose blocks wait for one another: on RSV_ETIMEOUT from
  *   rsv_sync_status() params, the Adam state and loss_out are those of an
- *   unfinished step, not to be used (check before rsv_mlp_mass is relied on).
+ *   unfinished step, not to be used.
  * rsv_mlp_mass: minv_out [T] = 1/m_t and, if m_out != NULL, m_out [T] = m_t,
  *   with m_t clamped to [1/s_u^2, A_t/s_eta^2 + 1/s_u^2 + (y_t^2/2) e^{-hbar_t}]
  *   (the observation precision, a floor of the posterior precision, and the
  *   diagonal of the Hessian of S at hbar; A_t = 1 + phi^2 inside, 1 at the
  *   ends, 1 - phi^2 if T = 1), so the mass cannot destabilise the leapfrog.
- *   y, hbar: [T] FP64 (the data and frozen mean the features came from). */
+ *   y, hbar: [T] FP64 (the data and frozen mean the features came from).
+ *   While a wait of this context that ran out is not yet reported by
+ *   rsv_sync_status(), both outputs are NaN: parameters of an unfinished
+ *   training never pass for a mass. */
 #define RSV_MLP_NPARAM 1761
 rsv_status rsv_welford_update(rsv_ctx* ctx, const float* x, int64_t n, int64_t T, int64_t count,
                               double* mean, double* m2, void* stream);

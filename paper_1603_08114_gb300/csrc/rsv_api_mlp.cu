@@ -112,7 +112,8 @@ rsv_status rsv_mlp_mass(rsv_ctx* c, const float* feat, int64_t T, const float* p
     if (T < 1) return fail(RSV_EINVAL, "T must be >= 1");
     if (!theta_ok(theta)) return fail(RSV_EINVAL, "invalid theta");
     cudaError_t e = counted(c, launch_mlp_mass, feat, T, params, y, hbar, to_dev(theta), log_scale,
-                            minv_out, m_out, (cudaStream_t)stream);
+                            (const int*)(c->ints.as<int>() + kStatus), minv_out, m_out,
+                            (cudaStream_t)stream);
     return e == cudaSuccess ? RSV_OK : cuda_fail(e, "mlp mass kernel");
 }
 

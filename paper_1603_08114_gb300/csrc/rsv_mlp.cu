@@ -671,6 +671,7 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
                                                   const double* __restrict__ y,
                                                   const double* __restrict__ hbar, ThetaD th,
                                                   const float* __restrict__ log_scale,
+                                                  const int* __restrict__ status,
                                                   float* __restrict__ minv, float* __restrict__ m_out)
 {
     __shared__ SParams sp;
@@ -688,6 +689,8 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
     const double in = (1.0 + th.phi * th.phi) / th.se2 + lo;
     const double end = (T == 1 ? 1.0 - th.phi * th.phi : 1.0) / th.se2 + lo;
     const float lof = (float)lo;
+    // parameters of a training that ended early give no mass
+    const float valid = (*status & ST_TIMEOUT) ? NAN : 1.f;
     for (int64_t base = ((int64_t)blockIdx.x * 4 + warp) * 32; base < T;
          base += (int64_t)gridDim.x * 128) {
         const int64_t s = base + lane;
@@ -720,8 +723,8 @@ __global__ void __launch_bounds__(128) k_mlp_mass(const float* __restrict__ feat
         if (act) {
             const double hi = (s == 0 || s == T - 1 ? end : in) + 0.5 * yv * yv * exp_neg(hv, s_exp);
             const float m = fminf(fmaxf(scale * (softplus_f(z) + EPS_M), lof), (float)hi);
-            minv[s] = 1.f / m;
-            if (m_out) m_out[s] = m;
+            minv[s] = valid / m;
+            if (m_out) m_out[s] = valid * m;
         }
     }
 }
@@ -1132,13 +1135,13 @@ cudaError_t launch_mlp_train(const float* feat, const float* target, int64_t T, 
 }
 
 cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, const double* y,
-                            const double* hbar, ThetaD th, const float* log_scale, float* minv,
-                            float* m_out, cudaStream_t st)
+                            const double* hbar, ThetaD th, const float* log_scale,
+                            const int* status, float* minv, float* m_out, cudaStream_t st)
 {
     int64_t g = (T + 127) / 128;
     if (g > 152 * 8) g = 152 * 8;
     k_mlp_mass<<<(int)(g < 1 ? 1 : g), 128, 0, st>>>(feat, T, params, y, hbar, th, log_scale,
-                                                      minv, m_out);
+                                                      status, minv, m_out);
     return cudaGetLastError();
 }
 

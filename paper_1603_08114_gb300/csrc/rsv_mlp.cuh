@@ -26,9 +26,10 @@ cudaError_t launch_mlp_train(const float* feat, const float* target, int64_t T, 
                              int batch, float* loss_out, const float* log_scale, bool capturing,
                              int num_sms, long long wait_limit, int* status, int64_t* launches,
                              cudaStream_t st);
+// NaN while *status holds ST_TIMEOUT.
 cudaError_t launch_mlp_mass(const float* feat, int64_t T, const float* params, const double* y,
-                            const double* hbar, ThetaD th, const float* log_scale, float* minv,
-                            float* m_out, cudaStream_t st);
+                            const double* hbar, ThetaD th, const float* log_scale,
+                            const int* status, float* minv, float* m_out, cudaStream_t st);
 cudaError_t launch_welford(const float* x, int64_t n, int64_t T, int64_t count, double* mean,
                            double* m2, cudaStream_t st);
 // partials: target_blocks() doubles (a block's sum each), counter: zero between launches.

@@ -74,9 +74,10 @@ class TrainedMass:
 
 def train_mass(ctx, y, lnrv, theta, mean, m2, count: int, steps: int = 2000, batch: int = 4096,
                lr: float = 1e-3, seed: int = 0, init_seed: int = 0) -> TrainedMass:
-    """Steps 2-5: target, features, Adam training, inverse mass.  Waits for
-    the training: one that ended early (a device-side wait beyond
-    rsv_set_wait_limit) raises RSV_ETIMEOUT instead of giving a mass."""
+    """Steps 2-5: target, features, Adam training, inverse mass.  After a training
+    that ended early (a device-side wait beyond rsv_set_wait_limit) the mass is
+    NaN until rsv_sync_status has reported it; where the program has set a limit
+    of its own, train_mass waits for the training and raises RSV_ETIMEOUT itself."""
     T = y.numel()
     hbar = torch.empty(T, dtype=torch.float64, device=y.device)
     log_s = torch.empty(1, dtype=torch.float32, device=y.device)
@@ -88,7 +89,8 @@ def train_mass(ctx, y, lnrv, theta, mean, m2, count: int, steps: int = 2000, bat
     losses = torch.empty(max(steps, 1), dtype=torch.float32, device=y.device)
     rsv.rsv_mlp_train(ctx, feat, target, params, am, av, 0, steps, batch, seed, lr,
                       loss_out=losses if steps else None, log_scale=log_s)
-    rsv.check_timeout(ctx)
+    if ctx.wait_limit:
+        rsv.check_timeout(ctx)
     minv = rsv.rsv_mlp_mass(ctx, feat, params, y, hbar, theta, log_scale=log_s)
     return TrainedMass(minv=minv, params=params, log_scale=log_s, losses=losses[:steps],
                        target=target,

@@ -138,6 +138,7 @@ class Context:
         # a non-finite dH found by a check in between (check_timeout), which the
         # next rsv_sync_status reports
         self.nonfinite = False
+        self.wait_limit = 0  # as set by rsv_set_wait_limit
         h = _P()
         _check(lib().rsv_create(ctypes.byref(h), int(device)))
         self.handle = h
@@ -180,6 +181,7 @@ def rsv_set_persistent(ctx: Context, enable: bool = True):
 def rsv_set_wait_limit(ctx: Context, cycles: int = 0):
     """Clock cycles a device-side wait may spin before RSV_ETIMEOUT (0: default)."""
     _check(lib().rsv_set_wait_limit(ctx.handle, int(cycles)))
+    ctx.wait_limit = int(cycles)
 
 
 def rsv_chain_schedule(ctx: Context, T: int, n_md: int, prec="mixed", with_mass=False):
