@@ -92,8 +92,8 @@ rsv_status rsv_sync_status(rsv_ctx* ctx, void* stream);
  * call that uses it fails with RSV_EINVAL).  A single series no longer than
  * `tile` is kept whole (it then needs only T <= threads * sites_per_thread).
  * All zero restores the automatic plan.  FP64 results do not depend on the
- * tiling (dH is summed free of order), mixed ones only through rounding (the
- * order of the sums). */
+ * tiling (dH is summed free of order as long as no site's energy reaches 2^28),
+ * mixed ones only through rounding (the order of the sums). */
 rsv_status rsv_set_schedule(rsv_ctx* ctx, int threads, int sites_per_thread, int64_t tile);
 /* rsv_set_persistent: 1 (the default) runs an rsv_hmc_chain call in RSV_MIXED
  * precision on the model without leverage as ONE persistent cooperative

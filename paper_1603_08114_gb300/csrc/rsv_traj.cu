@@ -149,8 +149,9 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
         // every term the same operations whatever the shape, their sum free
         // of the order they are taken in.
         int par = 0;
-        auto owned_energy = [&](double sign) {
+        auto owned_energy = [&](bool minus) {
             FixSum dE{0ull, 0ll, 0.0};
+            long long run = 0;
             double xL, xR;
             exchange(x[0], x[J - 1], xL, xR, s_edge + par * 2 * nw, nw);
             par ^= 1;
@@ -175,13 +176,14 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
                     if (s == 0) val = fma(0.5 * ie * st0 * x[j], x[j], val);
                     const double mi = MASS ? s_mi[j * NT + tid] : 1.0;
                     val = fma(0.5 * mi * p[j], p[j], val);
-                    fix_add(dE, sign * val);
+                    fix_term(dE, run, val, minus);
                 }
             }
+            fix_merge(dE, (unsigned long long)run << 14, run >> 50, 0.0);
             return fix_warp_sum(dE);
         };
         {   // (kept in shared memory through the steps)
-            const FixSum e0 = owned_energy(-1.0);
+            const FixSum e0 = owned_energy(true);
             if ((tid & 31) == 0) s_wpart[tid >> 5] = e0;
         }
 
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
                 }
             }
         }
-        const FixSum e1 = owned_energy(1.0);
+        const FixSum e1 = owned_energy(false);
         if ((tid & 31) == 0) fix_merge(s_wpart[tid >> 5], e1.lo, e1.hi, e1.big);
         __syncthreads();
         segment_decisions(A, v, s_wpart, s_wacc, &s_split);
