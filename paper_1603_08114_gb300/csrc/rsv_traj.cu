@@ -55,7 +55,7 @@ namespace {
 // a'[W] (with leverage y e^{-mu/2} instead), kc[W], and 1/m [W] with a mass.
 // Bound by the FP64 pipe.  Per site and leapfrog step 7 FP64 instructions (18
 // with the exponential on that pipe and both half drifts): a trajectory of
-// 2^20 sites and 100 steps 4.04 -> 1.46 ms.
+// 2^20 sites and 100 steps 4.04 -> 1.48 ms, the pipe 91 % busy.
 // ---------------------------------------------------------------------------
 template <int J, bool MASS, bool LEV>
 __global__ void __launch_bounds__(256, 1) k_traj_fp64(const TrajArgs A)
